@@ -130,29 +130,19 @@ struct Cfg {
   static_assert(BN % 32 == 0 && (BN / 32) * EPI_CHUNK <= RING, "epilogue chunks fit in the ring");
 };
 
-// Shared-memory matrix descriptor for a K-major operand tile with the 64-byte swizzle:
-// 64-byte rows, 8-row (512-byte) atoms stacked along M/N.  start >> 4 in bits 0-13, leading
-// byte offset >> 4 in 16-29 (unused by swizzled K-major layouts; 1), stride byte offset >> 4
-// (512) in 32-45, descriptor version 1 at bit 46, base offset 0, SWIZZLE_64B = 4 at 61-63.
-__device__ __forceinline__ uint64_t make_sdesc_sw64(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)1u << 16;
-  d |= (uint64_t)(512u >> 4) << 32;
-  d |= (uint64_t)1u << 46;
-  d |= (uint64_t)4u << 61;
-  return d;
-}
-
-// The same for the 128-byte swizzle: 128-byte rows, 8-row (1024-byte) atoms, SWIZZLE_128B = 2.
-__device__ __forceinline__ uint64_t make_sdesc_sw128(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)1u << 16;
-  d |= (uint64_t)(1024u >> 4) << 32;
-  d |= (uint64_t)1u << 46;
-  d |= (uint64_t)2u << 61;
-  return d;
+// Shared-memory matrix descriptor of a K-major operand tile, as two words.  Low: start >> 4 in bits 0-13,
+// leading byte offset >> 4 in 16-29 (unused by swizzled K-major layouts; 1).  High: stride byte offset >> 4
+// in bits 0-13 (8-row atoms stacked along M/N), descriptor version 1 at bit 14, base offset 0, swizzle mode
+// in bits 29-31.  64-byte rows: 512-byte atoms, SWIZZLE_64B = 4; 128-byte rows: 1024-byte atoms,
+// SWIZZLE_128B = 2.  Shared addresses stay below 256 KB, so a byte offset o adds o / 16 to the low word.
+__device__ __forceinline__ uint32_t sdesc_lo(uint32_t saddr) { return ((saddr & 0x3FFFFu) >> 4) | (1u << 16); }
+constexpr uint32_t kSdescHi64 = (512u >> 4) | (1u << 14) | (4u << 29);
+constexpr uint32_t kSdescHi128 = (1024u >> 4) | (1u << 14) | (2u << 29);
+// 1 in one lane of the warp, 0 in the others.
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+  return r;
 }
 
 // ---- PTX wrappers ----------------------------------------------------------------
@@ -242,23 +232,27 @@ __device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t ncols) {
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
+// One MMA, issued by the lane whose `leader` is not 0 with the rest of the warp beside it: the operands are
+// the same in every lane, so they stay in uniform registers, and come as the low words of their
+// shared-memory descriptors (sdesc_lo) plus the high word both share.  The warp that issues is bound by
+// its own instructions: with descriptors built in 64 bits by one diverged lane an MMA took at least 120
+// cycles whatever its width (a 128 x 128 x 16 one needs 64); in this form it runs at the tensor rate
+// (512 x 8192 by 3072, 128-wide tiles: 130 -> 93 us; 1024 x 3072 by 3072, 192-wide: 57 -> 48 us).
 template <class Md, uint32_t IDESC>
-__device__ __forceinline__ void mma(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
+__device__ __forceinline__ void mma(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t accumulate,
+                                    uint32_t leader) {
+#define SPL_MMA(KIND)                                                                                            \
+  asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %6, 0;\n\t" \
+               "mov.b64 da, {%1, %5};\n\tmov.b64 db, {%2, %5};\n\t"                                              \
+               "@q tcgen05.mma.cta_group::1." KIND " [%0], da, db, %3, p;\n\t}" ::"r"(d_tmem),                    \
+               "r"(a_lo), "r"(b_lo), "r"(IDESC), "r"(accumulate), "r"(hi), "r"(leader)                             \
+               : "memory")
   if constexpr (Md::kF16) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(IDESC), "r"(accumulate)
-        : "memory");
+    SPL_MMA("kind::f16");
   } else {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(IDESC), "r"(accumulate)
-        : "memory");
+    SPL_MMA("kind::tf32");
   }
+#undef SPL_MMA
 }
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
@@ -439,7 +433,7 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, float* __restrict__ out, con
   float* red = reinterpret_cast<float*>(smem);  // [BM][RED_STRIDE] staged accumulator, after the mainloop
   float* col_scale = reinterpret_cast<float*>(aux + 1024);  // [BN] FP16X3: 2^-e of the tile's W rows
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   // Linear tile id, M fastest: the CTAs that read the same weight tile run side by side and share it in L2.
   const int tile = tile_base + (int)blockIdx.x;
   const int64_t m0 = (int64_t)(tile % m_tiles) * BM, n0 = (int64_t)(tile / m_tiles) * BN;
@@ -478,7 +472,7 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, float* __restrict__ out, con
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
   if (warp == 0) {
     // ---------------- TMA producer: A_hi, A_lo, W_hi, W_lo ----------------
@@ -541,37 +535,47 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, float* __restrict__ out, con
         if (issued_mask & (1u << s)) mbar_wait(full_bar(s), (phase_mask >> s) & 1u, kDrainNs, nullptr);
     }
   } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
+    // ---------------- MMA issuer: the warp together, one lane issues ----------------
     bool ok = true;
+    const uint32_t leader = elect_one();
+    const uint32_t sd0 = sdesc_lo(smem_u32(smem));
+    int s = 0, in_seg = 0, seg = 0;
+    uint32_t ph = 0u;
     for (int kb = 0; kb < nk; ++kb) {
-      const int s = kb % STAGES;
-      const uint32_t ph = (uint32_t)(kb / STAGES) & 1u;
-      const int seg = kb / seg_len, in_seg = kb % seg_len;
       if (in_seg == 0 && seg >= 2) {  // P is free once the previous segment has been folded into R
         ok = __all_sync(0xffffffffu, mbar_wait(fold_bar, (uint32_t)(seg - 2) & 1u, kWaitNs, abort_flag));
         if (!ok) break;
       }
       ok = __all_sync(0xffffffffu, mbar_wait(full_bar(s), ph, kWaitNs, abort_flag));
       if (!ok) break;
-      if (lane == 0) {
-        tc_fence_after();
-        const uint32_t st = smem_u32(smem + (size_t)s * L::STAGE);
-        const uint32_t acc = tmem + (seg >= 1 ? L::P_OFF : 0u);
+      tc_fence_after();
+      const uint32_t sd = sd0 + (uint32_t)s * (L::STAGE >> 4);
+      const uint32_t acc = tmem + (seg >= 1 ? L::P_OFF : 0u);
 #pragma unroll
-        for (int kk = 0; kk < BK / Md::UMMA_K; ++kk) {
-          const uint32_t koff = kk * 32u;  // one instruction's K is 32 bytes of the 64-byte swizzled row
-          const uint32_t first = (in_seg == 0 && kk == 0) ? 0u : 1u;
-          mma<Md, L::IDESC>(acc, make_sdesc_sw64(st + L::A_LO + koff), make_sdesc_sw64(st + L::W_HI + koff), first);
-          mma<Md, L::IDESC>(acc, make_sdesc_sw64(st + L::A_HI + koff), make_sdesc_sw64(st + L::W_LO + koff), 1u);
-          mma<Md, L::IDESC>(acc, make_sdesc_sw64(st + L::A_HI + koff), make_sdesc_sw64(st + L::W_HI + koff), 1u);
-        }
+      for (int kk = 0; kk < BK / Md::UMMA_K; ++kk) {
+        const uint32_t k = sd + kk * 2u;  // one instruction's K is 32 bytes of the 64-byte swizzled row
+        const uint32_t first = (in_seg == 0 && kk == 0) ? 0u : 1u;
+        mma<Md, L::IDESC>(acc, k + (L::A_LO >> 4), k + (L::W_HI >> 4), kSdescHi64, first, leader);
+        mma<Md, L::IDESC>(acc, k + (L::A_HI >> 4), k + (L::W_LO >> 4), kSdescHi64, 1u, leader);
+        mma<Md, L::IDESC>(acc, k + (L::A_HI >> 4), k + (L::W_HI >> 4), kSdescHi64, 1u, leader);
+      }
+      const bool seg_end = in_seg == seg_len - 1 || kb == nk - 1;
+      if (leader) {
         mma_commit(empty_bar(s));  // stage reusable once these MMAs have read it
-        if (seg >= 1 && (in_seg == seg_len - 1 || kb == nk - 1)) mma_commit(seg_bar);  // P complete
+        if (seg >= 1 && seg_end) mma_commit(seg_bar);  // P complete
       }
       __syncwarp();
+      if (++in_seg == seg_len) {
+        in_seg = 0;
+        ++seg;
+      }
+      if (++s == STAGES) {
+        s = 0;
+        ph ^= 1u;
+      }
     }
     pdl_trigger();
-    if (lane == 0) {
+    if (leader) {
       if (!ok) {
         *abort_flag = 1;
         atomicOr(&g_device_status, kStatusTimeout);
@@ -781,7 +785,7 @@ tc_persistent_kernel(const __grid_constant__ TcMaps maps, float* __restrict__ ou
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(aux + 8 * (2 * STAGES + 5));
   volatile int* abort_flag = reinterpret_cast<volatile int*>(aux + 8 * (2 * STAGES + 5) + 8);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const int my_tiles = tiles > (int)blockIdx.x ? (tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
   const int nk = (int)ceil_div(K, BK);
   const int seg_len = chain > 0 && chain < nk ? chain : nk;  // k-blocks per segment
@@ -816,7 +820,7 @@ tc_persistent_kernel(const __grid_constant__ TcMaps maps, float* __restrict__ ou
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
   if (warp == 0) {
     // ---------------- TMA producer: the ring runs on across this CTA's tiles ----------------
@@ -861,7 +865,10 @@ tc_persistent_kernel(const __grid_constant__ TcMaps maps, float* __restrict__ ou
   } else if (warp == 1) {
     // ---------------- MMA issuer: tile i's segments into buffers i % 2 (R) and (i + 1) % 2 (P) ------
     bool ok = true;
-    uint32_t it = 0;
+    const uint32_t leader = elect_one();
+    const uint32_t sd0 = sdesc_lo(smem_u32(smem));
+    int st = 0;
+    uint32_t ph = 0u;
     uint32_t uses[2] = {0u, 0u};  // uses of each buffer so far
     for (int i = 0; i < my_tiles && ok; ++i) {
       for (int sg = 0; sg < nseg && ok; ++sg) {
@@ -873,36 +880,35 @@ tc_persistent_kernel(const __grid_constant__ TcMaps maps, float* __restrict__ ou
         tc_fence_after();
         const uint32_t acc = tmem + (uint32_t)b * ACC_COLS;
         const int kb0 = sg * seg_len, kb1 = std::min(nk, kb0 + seg_len);
-        for (int kb = kb0; kb < kb1; ++kb, ++it) {
-          const int st = (int)(it % STAGES);
-          const uint32_t ph = (it / STAGES) & 1u;
+        for (int kb = kb0; kb < kb1; ++kb) {
           ok = __all_sync(0xffffffffu, mbar_wait(full_bar(st), ph, kWaitNs, abort_flag));
           if (!ok) break;
-          if (lane == 0) {
-            tc_fence_after();
-            const uint32_t sa = smem_u32(smem + (size_t)st * L::STAGE);
+          tc_fence_after();
+          const uint32_t sd = sd0 + (uint32_t)st * (L::STAGE >> 4);
 #pragma unroll
-            for (int kk = 0; kk < BK / Md::UMMA_K; ++kk) {
-              const uint32_t koff = kk * 32u;
-              const uint32_t first = (kb == kb0 && kk == 0) ? 0u : 1u;
-              mma<Md, L::IDESC>(acc, make_sdesc_sw64(sa + L::A_LO + koff), make_sdesc_sw64(sa + L::W_HI + koff),
-                                first);
-              mma<Md, L::IDESC>(acc, make_sdesc_sw64(sa + L::A_HI + koff), make_sdesc_sw64(sa + L::W_LO + koff), 1u);
-              mma<Md, L::IDESC>(acc, make_sdesc_sw64(sa + L::A_HI + koff), make_sdesc_sw64(sa + L::W_HI + koff), 1u);
-            }
-            mma_commit(empty_bar(st));
+          for (int kk = 0; kk < BK / Md::UMMA_K; ++kk) {
+            const uint32_t k = sd + kk * 2u;
+            const uint32_t first = (kb == kb0 && kk == 0) ? 0u : 1u;
+            mma<Md, L::IDESC>(acc, k + (L::A_LO >> 4), k + (L::W_HI >> 4), kSdescHi64, first, leader);
+            mma<Md, L::IDESC>(acc, k + (L::A_HI >> 4), k + (L::W_LO >> 4), kSdescHi64, 1u, leader);
+            mma<Md, L::IDESC>(acc, k + (L::A_HI >> 4), k + (L::W_HI >> 4), kSdescHi64, 1u, leader);
           }
+          if (leader) mma_commit(empty_bar(st));
           __syncwarp();
+          if (++st == STAGES) {
+            st = 0;
+            ph ^= 1u;
+          }
         }
         if (!ok) break;
-        if (lane == 0) mma_commit(buf_full(b));  // this segment's sums are complete once these MMAs are
+        if (leader) mma_commit(buf_full(b));  // this segment's sums are complete once these MMAs are
         __syncwarp();
         ++uses[b];
       }
     }
     pdl_trigger();
     if (!ok) {
-      if (lane == 0) {
+      if (leader) {
         *abort_flag = 1;
         atomicOr(&g_device_status, kStatusTimeout);
         mma_commit(drain_bar);  // MMAs already issued finish before TMEM is released
@@ -1094,7 +1100,7 @@ tc_swap_kernel(const __grid_constant__ TcMaps maps, float* __restrict__ out, con
   volatile int* abort_flag = reinterpret_cast<volatile int*>(aux + L::AUX_BARS + 8);
   volatile int* last_flag = reinterpret_cast<volatile int*>(aux + L::AUX_BARS + 12);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const int64_t nkb = ceil_div(K, (int64_t)BK);
   const int64_t w_tiles = ceil_div(N, (int64_t)BM);
   const int64_t total = w_tiles * nkb;
@@ -1128,7 +1134,7 @@ tc_swap_kernel(const __grid_constant__ TcMaps maps, float* __restrict__ out, con
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   const int n_units = (int)(u1 - u0);
 
   if (warp == 0) {
@@ -1188,7 +1194,10 @@ tc_swap_kernel(const __grid_constant__ TcMaps maps, float* __restrict__ out, con
   } else if (warp == 1) {
     // ---------------- MMA issuer: chains of at most CH units, buffers alternating ----------------
     bool ok = true;
-    int j = 0, it = 0;  // unit of the run, chain of the run
+    const uint32_t leader = elect_one();
+    const uint32_t sd0 = sdesc_lo(smem_u32(smem));
+    int st = 0, it = 0;  // stage, chain of the run
+    uint32_t ph = 0u;
     for (int64_t u = u0; u < u1 && ok;) {
       const int64_t pe = std::min<int64_t>(u1, (u / nkb + 1) * nkb);  // end of the piece
       for (int64_t s = u; s < pe && ok;) {
@@ -1199,28 +1208,28 @@ tc_swap_kernel(const __grid_constant__ TcMaps maps, float* __restrict__ out, con
           if (!ok) break;
         }
         const uint32_t acc = tmem + (uint32_t)b * L::BUF;
-        for (int64_t v = s; v < se; ++v, ++j) {
-          const int st = j % STAGES;
-          const uint32_t ph = (uint32_t)(j / STAGES) & 1u;
+        for (int64_t v = s; v < se; ++v) {
           ok = __all_sync(0xffffffffu, mbar_wait(full_bar(st), ph, kWaitNs, abort_flag));
           if (!ok) break;
-          if (lane == 0) {
-            tc_fence_after();
-            const uint32_t sa = smem_u32(smem + (size_t)st * L::STAGE);
+          tc_fence_after();
+          const uint32_t sd = sd0 + (uint32_t)st * (L::STAGE >> 4);
 #pragma unroll
-            for (int kk = 0; kk < BK / 16; ++kk) {
-              const uint32_t koff = kk * 32u;  // one instruction's K is 32 bytes of the swizzled row
-              const uint32_t first = (v == s && kk == 0) ? 0u : 1u;
-              // W_hi x [x_lo; x_hi] (2 TN columns: hi*lo, then hi*hi), then W_lo x x_hi into the cross columns
-              mma<Fp16x3, L::IDESC_HI>(acc, make_sdesc_sw128(sa + L::W_HI + koff),
-                                       make_sdesc_sw128(sa + L::X_LO + koff), first);
-              mma<Fp16x3, L::IDESC_LO>(acc, make_sdesc_sw128(sa + L::W_LO + koff),
-                                       make_sdesc_sw128(sa + L::X_HI + koff), 1u);
-            }
+          for (int kk = 0; kk < BK / 16; ++kk) {
+            const uint32_t k = sd + kk * 2u;  // one instruction's K is 32 bytes of the swizzled row
+            const uint32_t first = (v == s && kk == 0) ? 0u : 1u;
+            // W_hi x [x_lo; x_hi] (2 TN columns: hi*lo, then hi*hi), then W_lo x x_hi into the cross columns
+            mma<Fp16x3, L::IDESC_HI>(acc, k + (L::W_HI >> 4), k + (L::X_LO >> 4), kSdescHi128, first, leader);
+            mma<Fp16x3, L::IDESC_LO>(acc, k + (L::W_LO >> 4), k + (L::X_HI >> 4), kSdescHi128, 1u, leader);
+          }
+          if (leader) {
             mma_commit(empty_bar(st));
             if (v == se - 1) mma_commit(buf_full(b));
           }
           __syncwarp();
+          if (++st == STAGES) {
+            st = 0;
+            ph ^= 1u;
+          }
         }
         ++it;
         s = se;
@@ -1228,7 +1237,7 @@ tc_swap_kernel(const __grid_constant__ TcMaps maps, float* __restrict__ out, con
       u = pe;
     }
     pdl_trigger();
-    if (lane == 0) {
+    if (leader) {
       if (!ok) {
         *abort_flag = 1;
         atomicOr(&g_device_status, kStatusTimeout);
