@@ -497,16 +497,19 @@ spl_status spl_test_tc_wait_timeout(float* out, const float* A, const spl_weight
  * product of M x K by N x K takes (seg_splits = 0), or a correction whose sums
  * follow a seg_splits-way split of K (the bank, seg_splits >= 1).  out[6]
  * (host) receives {tile width, ring KB, tiles of the unsplit launch, tiles of the
- * split launch, its K-split, 1 if the persistent kernel takes every tile (else
- * 0)}.  EINVAL for non-positive sizes, seg_splits outside
+ * split launch, its K-split, 1 if a persistent kernel takes every tile (else
+ * 0)}; ring KB 448 is the pair kernel (two SMs a 256-row tile), whose tiles are
+ * counted as 128-row ones and, for a correction, whose K-split is the one its
+ * segments follow.  EINVAL for non-positive sizes, seg_splits outside
  * [0, 8] or a NULL out.  No GPU work; needs a current CUDA device for the
  * occupancy queries. */
 spl_status spl_test_tc_shape(int64_t M, int64_t K, int64_t N, int64_t seg_splits, int64_t* out);
 
 /* Test hook (no counterpart in the paper): *out (host) = the number of clusters
  * of `cluster` CTAs (1..8) of the launch variant (tile_n, ring_kb) -- (256, 192),
- * (128, 224), (128, 96), (160, 224), (192, 224) or (224, 224) -- that can be
- * resident at once on the current device.
+ * (128, 224), (128, 96), (160, 224), (192, 224) or (224, 224), or the pair
+ * kernel's (256 | 224 | 192 | 160 | 128, 448) with cluster 1 (its CTAs) or 2 (its
+ * pairs) -- that can be resident at once on the current device.
  * EINVAL for another variant, cluster outside [1, 8] or a NULL out. */
 spl_status spl_test_tc_capacity(int64_t tile_n, int64_t ring_kb, int64_t cluster, int64_t* out);
 
@@ -523,7 +526,11 @@ spl_status spl_test_tc_capacity(int64_t tile_n, int64_t ring_kb, int64_t cluster
  * be 1 or seg_splits.  persistent != 0: every tile unsplit in the persistent
  * kernel (one CTA per SM looping over tiles, two TMEM accumulators; the result
  * equals the unsplit product bit for bit); it needs splits 1, seg_splits 0,
- * full_tiles 0, a one-CTA-per-SM variant and N % 4 == 0.  path is
+ * full_tiles 0, a one-CTA-per-SM variant and N % 4 == 0.  ring_kb 448 with
+ * tile_n 256, 224, 192, 160 or 128 is the pair kernel (FP16X3, persistent != 0,
+ * splits 1, full_tiles 0, N % 4 == 0, any seg_splits whose K ranges are single
+ * accumulation chains: EINVAL otherwise); its results equal the unsplit product's, or
+ * the seg_splits-way split's, bit for bit.  path is
  * SPL_PATH_TF32X3 or SPL_PATH_FP16X3.  Same operands, workspace and errors as
  * spl_masked_linear_unmask; EINVAL for another path or variant, full_tiles
  * outside [0, tiles], seg_splits outside [0, 8], a splits other than 1 or

@@ -23,6 +23,7 @@
 // split keeps fp32's exponent range) or FP32.  W is split once, offline; A is split by a pass before the product
 // into the workspace, so TMA lands every operand tile directly.
 //
+// Products from about 256 rows on run FP16X3 on SM pairs (gemm_pair.cuh).  The others:
 // Kernel shape (one CTA per 128 x BN output tile, 6 warps; BN = 256 with a 192 KB ring and
 // one CTA per SM, or BN = 128 with a 96 KB ring and two CTAs per SM, so that one CTA's
 // epilogue overlaps the other's mainloop):
@@ -238,19 +239,29 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 // its own instructions: with descriptors built in 64 bits by one diverged lane an MMA took at least 120
 // cycles whatever its width (a 128 x 128 x 16 one needs 64); in this form it runs at the tensor rate
 // (512 x 8192 by 3072, 128-wide tiles: 130 -> 93 us; 1024 x 3072 by 3072, 192-wide: 57 -> 48 us).
-template <class Md, uint32_t IDESC>
+// CTAS = 2: the pair's MMA.  COLL: what it does with the A operand in the tensor core's collector buffer --
+// nothing, keep it for the next MMA, or use (and drop) the one the MMA before kept.
+enum Collect { kCollNone = 0, kCollFill = 1, kCollUse = 2 };
+template <class Md, uint32_t IDESC, int CTAS = 1, int COLL = kCollNone>
 __device__ __forceinline__ void mma(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t accumulate,
                                     uint32_t leader) {
-#define SPL_MMA(KIND)                                                                                            \
+  static_assert(CTAS == 1 ? COLL == kCollNone : Md::kF16, "pairs and the collector: fp16 pairs only");
+#define SPL_MMA(GROUP_KIND)                                                                                      \
   asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %6, 0;\n\t" \
                "mov.b64 da, {%1, %5};\n\tmov.b64 db, {%2, %5};\n\t"                                              \
-               "@q tcgen05.mma.cta_group::1." KIND " [%0], da, db, %3, p;\n\t}" ::"r"(d_tmem),                    \
+               "@q tcgen05.mma.cta_group::" GROUP_KIND " [%0], da, db, %3, p;\n\t}" ::"r"(d_tmem),                \
                "r"(a_lo), "r"(b_lo), "r"(IDESC), "r"(accumulate), "r"(hi), "r"(leader)                             \
                : "memory")
-  if constexpr (Md::kF16) {
-    SPL_MMA("kind::f16");
+  if constexpr (CTAS == 2 && COLL == kCollFill) {
+    SPL_MMA("2.kind::f16.collector::a::fill");
+  } else if constexpr (CTAS == 2 && COLL == kCollUse) {
+    SPL_MMA("2.kind::f16.collector::a::lastuse");
+  } else if constexpr (CTAS == 2) {
+    SPL_MMA("2.kind::f16");
+  } else if constexpr (Md::kF16) {
+    SPL_MMA("1.kind::f16");
   } else {
-    SPL_MMA("kind::tf32");
+    SPL_MMA("1.kind::tf32");
   }
 #undef SPL_MMA
 }
@@ -1390,6 +1401,8 @@ tc_swap_kernel(const __grid_constant__ TcMaps maps, float* __restrict__ out, con
   }
 }
 
+#include "gemm_pair.cuh"
+
 // ---- host side: tensor maps ------------------------------------------------------
 using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                    const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -1454,6 +1467,20 @@ bool set_smem_attr_persistent() {
   return true;
 }
 
+template <int BN>
+bool set_smem_attr_pair() {
+  static bool done[64] = {false};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+  if (!done[dev]) {
+    if (cudaFuncSetAttribute(tc_pair_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)PairCfg<BN>::SMEM) != cudaSuccess)
+      return false;
+    done[dev] = true;
+  }
+  return true;
+}
+
 template <int TN>
 bool set_smem_attr_swap() {
   static bool done[64] = {false};
@@ -1479,24 +1506,21 @@ int swap_width_index(int64_t tokens) {
   return kSwapWidths - 1;
 }
 
-// The launch variants: tile width, ring size, CTAs per SM, and the cost constants of the
-// launch model below.  Cost of one round of co-resident CTAs, in units of K: F + f s + b K / s
-// (F: setup, pipeline fill and epilogue of a CTA; f: the cluster reduction per rank; b: the
-// mainloop per K element, relative to the 256-wide tile with the 192 KB ring), fitted to a sweep
-// of every variant, split and whole-wave form over the eight Llama and Qwen projections at 128,
-// 512, 1024, 2048 and 4096 rows on GB300: the shapes it picks (ties going to the earlier variant,
-// as below) are within 0.5% of the best measured, on average over the 40 cases.  A k-step of a narrower tile costs almost as much as
-// one of a 256-wide tile (b ~ 1 for every width), so the narrower tiles win only where they fill
-// a wave that the 256-wide tiles leave part empty (e.g. 512 x 3072 by 3072: 64 tiles of 192
-// columns in clusters of 2 instead of 48 of 256).
+// The launch variants: tile width, ring size, CTAs per SM, and the cost constants of the launch model
+// below, in us: a round of co-resident CTAs takes F + b K / s (F: setup, pipeline fill, epilogue and
+// cluster reduction; b: the mainloop per 1000 elements of K on FP16X3; TF32X3 takes two k-blocks where
+// FP16X3 takes one).  Fitted to a sweep of every variant, split, persistent and pair form over the eight
+// Llama and Qwen projections at 61 to 2048 rows on GB300 (64 shapes): the picks are within 0.8% of the
+// best form measured on average, 8% at worst (61 rows by 19456 outputs, where HBM is the bound and the
+// model does not see it); the model before the MMA issue was fixed was 10% off on average.
 struct Variant {
   int bn, rk, cps;
-  double F, f, b;
+  double F, b;
 };
 constexpr int kVariants = 6;
-constexpr Variant kVariant[kVariants] = {{256, 192, 1, 500.0, 20.0, 1.0},   {128, 224, 1, 300.0, 20.0, 1.05},
-                                         {128, 96, 2, 250.0, 20.0, 0.95},   {160, 224, 1, 250.0, 20.0, 1.05},
-                                         {192, 224, 1, 300.0, 20.0, 1.0},   {224, 224, 1, 550.0, 20.0, 0.97}};
+constexpr Variant kVariant[kVariants] = {{256, 192, 1, 8.22, 16.08}, {128, 224, 1, 6.26, 10.58},
+                                         {128, 96, 2, 7.33, 17.81},  {160, 224, 1, 6.78, 11.62},
+                                         {192, 224, 1, 7.28, 12.78}, {224, 224, 1, 7.32, 14.40}};
 
 // Co-resident clusters of s CTAs of variant v on the current device; clusters must fit inside
 // one GPC, so this is not simply (SMs x CTAs per SM) / s.  Both encodings use the same shared
@@ -1542,35 +1566,95 @@ int max_active_clusters(int v, int s, int sms) {
   return c;
 }
 
-// Launch shape: a variant, then either one launch with every tile's K split s ways over a
-// cluster, or whole waves of unsplit tiles followed by the remaining tiles split (so the last
-// wave is not mostly idle).  Cost of a launch in units of K: rounds x (F + f s + b K / s), rounds
-// counting co-resident CTAs.  At least 256 of K per CTA; ties go to the earlier variant and to
-// fewer splits.
+// Launch shape: a variant, then either one launch with every tile's K split s ways over a cluster, or
+// whole waves of unsplit tiles followed by the remaining tiles split (so the last wave is not mostly
+// idle), or one persistent launch, on single SMs or on SM pairs.  At least 256 of K per CTA; ties go to
+// the earlier variant and to fewer splits.
 struct TcShape {
   int v;
   int64_t full_tiles;  // tiles of the first, unsplit launch (whole waves)
   int64_t rest_tiles;  // tiles of the second launch
   int rest_splits;
-  double cost;
+  double cost;              // us
   bool persistent = false;  // one launch of tc_persistent_kernel over every tile (unsplit)
+  int pair = -1;            // >= 0: width index of tc_pair_kernel, one launch over every tile (unsplit)
 };
 
-// Cost of the persistent form: the first prologue and the last epilogue (F) once, then per tile of
-// the busiest CTA its mainloop and a small hand-over (kPersistentTile, in units of K).  With it the
-// shapes picked over the eight projections at 512 to 4096 rows (persistent, split and whole-wave
-// forms all timed) are within 0.16% of the best measured on average; the persistent form saves 4-7%
-// on shapes of several waves (e.g. 2048 x 2560 by 19456: 386.5 against 412.8 us).
-constexpr double kPersistentTile = 60.0;
+// Widths of the pair kernel's 256-row tiles (FP16X3) and their cost in us: F once, then per tile of the
+// busiest pair b K plus h (the part of a tile's hand-over and epilogue that its successor does not hide).
+// Fitted with the variants above.  A pair beats two single SMs from about 256 rows on: its tile needs
+// 32 KB a k-block per SM where a 128 x 256 tile needs 48, so the tensor pipe is not kept waiting
+// (256-wide: 13.0 against 16.1 us per 1000 of K).  Times at 1024 rows (with the split of A): 3072 by 16384
+// 229 -> 179 us, 3072 by 3072 48 -> 44 us, 8192 by 3072 122 -> 101 us; at 4096 rows 3072 by 16384
+// 871 -> 682 us, where it runs at the power limit (1.8 PFLOP/s of fp16).
+struct PairWidth {
+  int bn;
+  double F, h, b;
+};
+constexpr int kPairs = 5;
+constexpr PairWidth kPair[kPairs] = {{256, 5.50, 6.96, 13.00},
+                                     {224, 5.33, 3.16, 12.38},
+                                     {192, 4.70, 1.15, 11.25},
+                                     {160, 4.68, 0.00, 10.28},
+                                     {128, 2.68, 1.87, 7.57}};
+constexpr int kPairRingKb = 448;  // how the test hooks name the pair variants: two SMs' shared memory
 
-double launch_cost(int v, int64_t tiles, int64_t K, int s, int sms) {
-  if (tiles <= 0) return 0.0;
-  const int64_t capacity = (int64_t)max_active_clusters(v, s, sms) * s;
-  const int64_t rounds = ceil_div(tiles * s, capacity);
-  return (double)rounds * (kVariant[v].F + kVariant[v].f * s + kVariant[v].b * (double)K / (double)s);
+// Co-resident pairs of the pair kernel (clusters of two CTAs, one CTA per SM).
+template <int BN>
+int active_pairs() {
+  static int cache[64] = {0};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return std::max(1, device_sm_count() / 2);
+  if (cache[dev] == 0) {
+    int n = 0;
+    cudaLaunchConfig_t cfg;
+    std::memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3(2, 1, 1);
+    cfg.blockDim = dim3(PAIR_THREADS, 1, 1);
+    cfg.dynamicSmemBytes = PairCfg<BN>::SMEM;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (!set_smem_attr_pair<BN>() ||
+        cudaOccupancyMaxActiveClusters(&n, tc_pair_kernel<BN>, &cfg) != cudaSuccess)
+      n = 0;
+    cudaGetLastError();
+    cache[dev] = n > 0 ? n : std::max(1, device_sm_count() / 2);
+  }
+  return cache[dev];
 }
 
-TcShape tc_shape_for(int v, int64_t M, int64_t K, int64_t N, int sms) {
+int pairs_of(int w) {
+  switch (w) {
+    case 0: return active_pairs<kPair[0].bn>();
+    case 1: return active_pairs<kPair[1].bn>();
+    case 2: return active_pairs<kPair[2].bn>();
+    case 3: return active_pairs<kPair[3].bn>();
+    default: return active_pairs<kPair[4].bn>();
+  }
+}
+
+// Cost in us of the single-SM persistent form: F once, then per tile of the busiest CTA its mainloop and a
+// hand-over.  It is left where a 256-row tile would be half empty (up to 128 rows of several waves) and for
+// TF32X3.
+constexpr double kPersistentTile = 6.73;
+
+double k_cost(double b, int64_t K, bool f16) { return b * 1e-3 * (double)K * (f16 ? 1.0 : 2.0); }
+
+double launch_cost(int v, int64_t tiles, int64_t K, int s, int sms, bool f16) {
+  if (tiles <= 0) return 0.0;
+  // clusters of 3, 5 or 7 CTAs: one fewer fits than the occupancy query says (exactly full grids of them
+  // took a second round: 256 x 9728 by 2560, 28 clusters of 5, 62 us against 38 for 24 of 5)
+  int64_t clusters = max_active_clusters(v, s, sms);
+  if (s > 1 && (s & 1) != 0 && clusters > 1) --clusters;
+  return (double)ceil_div(tiles, clusters) * (kVariant[v].F + k_cost(kVariant[v].b, K, f16) / (double)s);
+}
+
+TcShape tc_shape_for(int v, int64_t M, int64_t K, int64_t N, int sms, bool f16) {
   // the persistent epilogue stores whole float4s: output rows of whole 16-byte units (a launch whose
   // pointers are not 16-byte aligned runs the same tiles unsplit in tc_gemm_kernel: the same sums)
   const bool persistent_ok = (N & 3) == 0;
@@ -1578,7 +1662,7 @@ TcShape tc_shape_for(int v, int64_t M, int64_t K, int64_t N, int sms) {
   const int max_s = (int)std::max<int64_t>(1, std::min<int64_t>(MAX_CLUSTER, K / 256));
   TcShape best{v, 0, tiles, 1, 1e300};
   for (int s = 1; s <= max_s; ++s) {
-    const double c = launch_cost(v, tiles, K, s, sms);
+    const double c = launch_cost(v, tiles, K, s, sms, f16);
     if (c < best.cost * (1.0 - 1e-9)) best = TcShape{v, 0, tiles, s, c};
   }
   const int64_t wave = max_active_clusters(v, 1, sms);
@@ -1587,14 +1671,14 @@ TcShape tc_shape_for(int v, int64_t M, int64_t K, int64_t N, int sms) {
   const int64_t m_tiles = ceil_div(M, BM);
   const int64_t full = (tiles / wave) * wave / m_tiles * m_tiles, rest = tiles - full;
   if (full > 0 && rest > 0) {
-    const double cf = launch_cost(v, full, K, 1, sms);
+    const double cf = launch_cost(v, full, K, 1, sms, f16);
     for (int s = 1; s <= max_s; ++s) {
-      const double c = cf + launch_cost(v, rest, K, s, sms);
+      const double c = cf + launch_cost(v, rest, K, s, sms, f16);
       if (c < best.cost * (1.0 - 1e-9)) best = TcShape{v, full, rest, s, c};
     }
   }
   if (persistent_ok && kVariant[v].cps == 1 && tiles > wave) {  // more than one wave of unsplit tiles
-    const double c = kVariant[v].F + (double)ceil_div(tiles, wave) * (kVariant[v].b * (double)K + kPersistentTile);
+    const double c = kVariant[v].F + (double)ceil_div(tiles, wave) * (k_cost(kVariant[v].b, K, f16) + kPersistentTile);
     if (c < best.cost * (1.0 - 1e-9)) {
       best = TcShape{v, 0, tiles, 1, c};
       best.persistent = true;
@@ -1603,32 +1687,57 @@ TcShape tc_shape_for(int v, int64_t M, int64_t K, int64_t N, int sms) {
   return best;
 }
 
+// The cheapest pair form, if it beats `best` (FP16X3, output rows of whole 16-byte units): M and N in tiles
+// of the widths, every one unsplit.  rest_tiles counts 128-row tiles, as the other forms do.
+void consider_pairs(TcShape& best, int64_t M, int64_t K, int64_t N) {
+  if ((N & 3) != 0) return;
+  for (int w = 0; w < kPairs; ++w) {
+    const int64_t cols = ceil_div(N, (int64_t)kPair[w].bn), tiles = ceil_div(M, (int64_t)256) * cols;
+    const double c =
+        kPair[w].F + (double)ceil_div(tiles, (int64_t)pairs_of(w)) * (k_cost(kPair[w].b, K, true) + kPair[w].h);
+    if (c < best.cost * (1.0 - 1e-9)) {
+      best = TcShape{0, 0, ceil_div(M, BM) * cols, 1, c};
+      best.pair = w;
+    }
+  }
+}
+
+// k-blocks of a rank of an s-way split of K.
+template <class Md>
+int rank_blocks_of(int64_t K, int s) {
+  return (int)(round_up(ceil_div(K, s), Md::BK) / Md::BK);
+}
+
 // Shape of a correction whose sums must follow a seg_splits-way split of K (the bank): whole
 // waves of unsplit tiles that fold the K ranges in TMEM (segmented mode), then the remaining
 // tiles with K split seg_splits ways over a cluster, whose rank-order sum is the same fold; or
-// every tile segmented.  The cheapest variant and form.
-TcShape tc_bank_shape(int64_t M, int64_t K, int64_t N, int seg_splits, int sms) {
+// every tile segmented, on single SMs or on pairs.  The cheapest variant and form.
+TcShape tc_bank_shape(int64_t M, int64_t K, int64_t N, int seg_splits, int sms, bool f16) {
   TcShape best{0, 0, 0, 1, 1e300};
   for (int v = 0; v < kVariants; ++v) {
     const int64_t tiles = ceil_div(M, BM) * ceil_div(N, kVariant[v].bn);
-    const double c = launch_cost(v, tiles, K, 1, sms);
+    const double c = launch_cost(v, tiles, K, 1, sms, f16);
     if (c < best.cost * (1.0 - 1e-9)) best = TcShape{v, 0, tiles, 1, c};
     if (seg_splits < 2 || seg_splits > MAX_CLUSTER) continue;
     const int64_t wave = max_active_clusters(v, 1, sms);
     const int64_t full = (tiles / wave) * wave, rest = tiles - full;
     if (rest == 0) continue;
-    const double c2 = launch_cost(v, full, K, 1, sms) + launch_cost(v, rest, K, seg_splits, sms);
+    const double c2 = launch_cost(v, full, K, 1, sms, f16) + launch_cost(v, rest, K, seg_splits, sms, f16);
     if (c2 < best.cost * (1.0 - 1e-9)) best = TcShape{v, full, rest, seg_splits, c2};
   }
+  // segments longer than a chain belong to ranks that fold chains of their own: only a split reproduces them
+  if (f16 && (seg_splits == 1 || rank_blocks_of<Fp16x3>(K, seg_splits) <= kChainBlocks))
+    consider_pairs(best, M, K, N);
   return best;
 }
 
-TcShape tc_shape(int64_t M, int64_t K, int64_t N, int sms) {
-  TcShape best = tc_shape_for(0, M, K, N, sms);
+TcShape tc_shape(int64_t M, int64_t K, int64_t N, int sms, bool f16) {
+  TcShape best = tc_shape_for(0, M, K, N, sms, f16);
   for (int v = 1; v < kVariants; ++v) {
-    const TcShape t = tc_shape_for(v, M, K, N, sms);
+    const TcShape t = tc_shape_for(v, M, K, N, sms, f16);
     if (t.cost < best.cost * (1.0 - 1e-9)) best = t;
   }
+  if (f16) consider_pairs(best, M, K, N);
   return best;
 }
 
@@ -1652,7 +1761,7 @@ spl_status launch_tc(const LinearArgs& a, const uint16_t* a_hi, const uint16_t* 
   if (seg_splits == 1) {
     seg_blocks = chain_segments<Md>(a.K);
   } else if (seg_splits > 1) {
-    const int rank_blocks = (int)(round_up(ceil_div(a.K, seg_splits), Md::BK) / Md::BK);
+    const int rank_blocks = rank_blocks_of<Md>(a.K, seg_splits);
     if (rank_blocks <= kChainBlocks) {
       seg_blocks = rank_blocks;
     } else {  // every tile as the online launch ran it: split seg_splits ways, each rank folding its chains
@@ -1741,6 +1850,56 @@ spl_status launch_tc(const LinearArgs& a, const uint16_t* a_hi, const uint16_t* 
   return launch(shape.rest_tiles, shape.full_tiles, shape.rest_splits, shape.rest_splits > 1 ? 0 : seg_blocks);
 }
 
+// Every tile of the product on the pair kernel, segments of `chain` k-blocks.
+template <int BN>
+spl_status launch_pair_bn(const LinearArgs& a, const uint16_t* a_hi, const uint16_t* a_lo, const int* a_exp, int chain) {
+  using L = PairCfg<BN>;
+  if (!set_smem_attr_pair<BN>()) return SPL_ECUDA;
+  if ((a.N & 3) != 0 || !aligned16(a.out) || (a.c && !aligned16(a.c))) return SPL_EALIGN;  // whole 16-byte units
+  const int64_t m_tiles = ceil_div(a.M, (int64_t)256), tiles = m_tiles * ceil_div(a.N, (int64_t)BN);
+  if (tiles > 0x3fffffffLL) return SPL_ESHAPE;
+  TcMaps maps;
+  std::memset(&maps, 0, sizeof(maps));
+  const int64_t c_rows = a.c ? std::min<int64_t>(a.c_rows, a.M) : 0;
+  if (!make_map(&maps.a_hi, a_hi, true, a.M, a.K, L::BK, 128, CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !make_map(&maps.a_lo, a_lo, true, a.M, a.K, L::BK, 128, CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !make_map(&maps.w_hi, a.w_h16, true, a.N, a.K, L::BK, BN / 2, CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !make_map(&maps.w_lo, a.w_l16, true, a.N, a.K, L::BK, BN / 2, CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !make_map(&maps.y, a.out, false, a.M, a.N, 32, 32, CU_TENSOR_MAP_SWIZZLE_128B) ||
+      (c_rows > 0 && !make_map(&maps.c, a.c, false, c_rows, a.N, 32, 32, CU_TENSOR_MAP_SWIZZLE_128B)))
+    return SPL_ECUDA;
+  const int64_t pairs = std::min<int64_t>(tiles, active_pairs<BN>());
+  cudaLaunchConfig_t cfg;
+  std::memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3((unsigned)(2 * pairs), 1, 1);
+  cfg.blockDim = dim3(PAIR_THREADS, 1, 1);
+  cfg.dynamicSmemBytes = L::SMEM;
+  cfg.stream = a.stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, tc_pair_kernel<BN>, maps, a_exp, (const int*)a.w_exp, a.M, a.K, a.N,
+                                           (int)tiles, (int)m_tiles, chain, c_rows);
+  note_launches(1);
+  return e == cudaSuccess ? SPL_OK : SPL_ECUDA;
+}
+
+spl_status launch_pair(const LinearArgs& a, const uint16_t* hi, const uint16_t* lo, const int* a_exp, int w, int chain) {
+  switch (w) {
+    case 0: return launch_pair_bn<kPair[0].bn>(a, hi, lo, a_exp, chain);
+    case 1: return launch_pair_bn<kPair[1].bn>(a, hi, lo, a_exp, chain);
+    case 2: return launch_pair_bn<kPair[2].bn>(a, hi, lo, a_exp, chain);
+    case 3: return launch_pair_bn<kPair[3].bn>(a, hi, lo, a_exp, chain);
+    default: return launch_pair_bn<kPair[4].bn>(a, hi, lo, a_exp, chain);
+  }
+}
+
 template <class Md>
 spl_status launch_variant(const LinearArgs& a, const uint16_t* hi, const uint16_t* lo, const int* a_exp,
                           const TcShape& shape, int skip_kblock, int seg_splits) {
@@ -1827,8 +1986,10 @@ spl_status launch_swap(const LinearArgs& a, const uint16_t* x_hi, const uint16_t
 // swap_w >= 0: the swapped kernel with that token-tile width index and swap_s CTAs per token tile
 // (0: the library's count, which depends on K and N only, so a bank of any width meets the online
 // product's runs).
+// pair_w >= 0: every tile on the pair kernel of that width index (FP16X3).
 spl_status run_tc_impl(const LinearArgs& a, int skip_kblock, int forced_v, int forced_splits, int seg_splits = 0,
-                       int64_t forced_full = 0, bool forced_persistent = false, int swap_w = -1, int swap_s = 0) {
+                       int64_t forced_full = 0, bool forced_persistent = false, int swap_w = -1, int swap_s = 0,
+                       int pair_w = -1) {
   const int cc = device_cc();
   if (cc != 100 && cc != 103) return SPL_EUNSUPPORTED;
   const bool f16 = a.path == SPL_PATH_FP16X3;
@@ -1890,12 +2051,20 @@ spl_status run_tc_impl(const LinearArgs& a, int skip_kblock, int forced_v, int f
     shape = TcShape{forced_v, forced_full, tiles - forced_full, forced_splits, 0.0};
     shape.persistent = forced_persistent;
   } else if (seg_splits > 0) {
-    shape = tc_bank_shape(a.M, a.K, a.N, seg_splits, device_sm_count());
+    shape = tc_bank_shape(a.M, a.K, a.N, seg_splits, device_sm_count(), f16);
   } else {
-    shape = tc_shape(a.M, a.K, a.N, device_sm_count());
+    shape = tc_shape(a.M, a.K, a.N, device_sm_count(), f16);
   }
+  if (pair_w >= 0) shape.pair = pair_w;
   const uint16_t* hi = static_cast<const uint16_t*>(a_hi);
   const uint16_t* lo = static_cast<const uint16_t*>(a_lo);
+  if (f16 && shape.pair >= 0 && skip_kblock < 0) {
+    // segments at the online split's K ranges where each is one chain, else chains of kChainBlocks
+    int chain = kChainBlocks;
+    if (seg_splits > 1) chain = rank_blocks_of<Fp16x3>(a.K, seg_splits);
+    if (chain > kChainBlocks) return SPL_EINVAL;
+    return launch_pair(a, hi, lo, a_exp, shape.pair, chain);
+  }
   return f16 ? launch_variant<Fp16x3>(a, hi, lo, a_exp, shape, skip_kblock, seg_splits)
              : launch_variant<Tf32x3>(a, hi, lo, a_exp, shape, skip_kblock, seg_splits);
 }
@@ -1917,7 +2086,7 @@ Plan plan_tc(int64_t M, int64_t K, int64_t N, int sms, spl_path path) {
     p.splits = 1;  // runs of k-blocks, partial tiles summed through the workspace
     p.ws_partials = tc_partial_bytes(M, K, N, M, path);
   } else {
-    const TcShape t = tc_shape(M, K, N, sms);
+    const TcShape t = tc_shape(M, K, N, sms, path == SPL_PATH_FP16X3);
     p.splits = t.rest_splits;  // partials are reduced through distributed shared memory
   }
   p.k_per_split = ceil_div(K, p.splits);
@@ -1944,9 +2113,9 @@ bool tc_uniform_shape(int64_t M, int64_t K, int64_t N, spl_path path, int* varia
     *splits = 1;
     return true;
   }
-  const TcShape t = tc_shape(M, K, N, device_sm_count());
+  const TcShape t = tc_shape(M, K, N, device_sm_count(), path == SPL_PATH_FP16X3);
   if (t.full_tiles > 0 && t.rest_tiles > 0) return false;
-  *variant = t.v;
+  *variant = t.pair >= 0 ? kVariants + t.pair : t.v;
   *splits = t.full_tiles > 0 ? 1 : t.rest_splits;
   return true;
 }
@@ -1984,13 +2153,14 @@ extern "C" spl_status spl_test_tc_shape(int64_t M, int64_t K, int64_t N, int64_t
   using namespace spl;
   if (!out || M <= 0 || K <= 0 || N <= 0 || seg_splits < 0 || seg_splits > MAX_CLUSTER) return SPL_EINVAL;
   const int sms = device_sm_count();
-  const TcShape t = seg_splits > 0 ? tc_bank_shape(M, K, N, (int)seg_splits, sms) : tc_shape(M, K, N, sms);
-  out[0] = kVariant[t.v].bn;
-  out[1] = kVariant[t.v].rk;
+  const TcShape t =
+      seg_splits > 0 ? tc_bank_shape(M, K, N, (int)seg_splits, sms, true) : tc_shape(M, K, N, sms, true);
+  out[0] = t.pair >= 0 ? kPair[t.pair].bn : kVariant[t.v].bn;
+  out[1] = t.pair >= 0 ? kPairRingKb : kVariant[t.v].rk;
   out[2] = t.full_tiles;
   out[3] = t.rest_tiles;
-  out[4] = t.rest_splits;
-  out[5] = t.persistent ? 1 : 0;
+  out[4] = t.pair >= 0 && seg_splits > 0 ? seg_splits : t.rest_splits;  // a bank on pairs folds that split's ranges
+  out[5] = t.persistent || t.pair >= 0 ? 1 : 0;
   return SPL_OK;
 }
 
@@ -2003,6 +2173,11 @@ extern "C" spl_status spl_test_tc_capacity(int64_t tile_n, int64_t ring_kb, int6
   for (int v = 0; v < kVariants; ++v)
     if (kVariant[v].bn == tile_n && kVariant[v].rk == ring_kb) {
       *out = max_active_clusters(v, (int)cluster, device_sm_count());
+      return SPL_OK;
+    }
+  for (int w = 0; w < kPairs; ++w)
+    if (kPair[w].bn == tile_n && ring_kb == kPairRingKb && cluster <= 2) {
+      *out = (int64_t)pairs_of(w) * (cluster == 1 ? 2 : 1);
       return SPL_OK;
     }
   return SPL_EINVAL;
@@ -2019,10 +2194,21 @@ extern "C" spl_status spl_test_tc_product(float* out, const float* A, const spl_
   using namespace spl;
   if (!out || !A || !W || !W->w || M <= 0 || N <= 0 || K <= 0) return SPL_EINVAL;
   if (path != SPL_PATH_TF32X3 && path != SPL_PATH_FP16X3) return SPL_EINVAL;
-  int v = -1;
+  int v = -1, pair = -1;
   for (int i = 0; i < kVariants; ++i)
     if (kVariant[i].bn == tile_n && kVariant[i].rk == ring_kb) v = i;
-  if (v < 0) return SPL_EINVAL;
+  for (int i = 0; i < kPairs; ++i)
+    if (kPair[i].bn == tile_n && ring_kb == kPairRingKb) pair = i;
+  if (v < 0 && pair < 0) return SPL_EINVAL;
+  if (pair >= 0) {  // every tile unsplit on the pair kernel
+    if (path != SPL_PATH_FP16X3 || splits != 1 || full_tiles != 0 || !persistent || seg_splits < 0 ||
+        seg_splits > MAX_CLUSTER || (N & 3) != 0)
+      return SPL_EINVAL;
+    if ((K & 3) != 0) return SPL_EALIGN;
+    if (!aligned16(out) || !aligned16(A) || (C && !aligned16(C))) return SPL_EALIGN;
+    const LinearArgs args = make_args(out, A, *W, C, M, K, N, workspace, workspace_bytes, stream, path);
+    return run_tc_impl(args, -1, 0, 1, seg_splits, 0, false, -1, 0, pair);
+  }
   if (splits < 1 || splits > MAX_CLUSTER) return SPL_ESHAPE;
   if ((K & 3) != 0) return SPL_EALIGN;
   if (!aligned16(out) || !aligned16(A) || (C && !aligned16(C))) return SPL_EALIGN;
