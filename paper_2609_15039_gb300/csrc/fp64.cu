@@ -7,6 +7,10 @@
 // binary64, the correction W eta is kept in binary64 and subtracted in binary64; only Y is rounded
 // to fp32 at the end.
 //
+// Products of a few rows on run as exact slices on the tensor cores (gemm_f64.cuh, by the rule in fp64.cuh),
+// whose result is closer to the exact sum than a binary64 sum's.  The kernels here take the rest, on the FP64
+// pipe.
+//
 // Kernel: the decode kernel's structure in binary64 -- a 256-thread block owns 16 rows of W over
 // a K-slice, stages MT (1, 2, 4 or 8) rows of the left operand of that slice in shared memory (as
 // binary64), streams W once and keeps 2 x MT binary64 partial sums per lane, reduced across the
@@ -17,6 +21,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "fp64.cuh"
 
 namespace spl {
 namespace {
@@ -39,30 +44,7 @@ __device__ __forceinline__ double2 load_a2<double>(const double* p) {
   return __ldg(reinterpret_cast<const double2*>(p));
 }
 
-// Final value of an output (one split, or after the split-order reduction):
-//   kOut64  out64 = acc (the correction C, binary64)
-//   kUnmask out32 = fl32(acc - c)
-//   kSlalom out32 = ((acc - c) mod q, taken in (-q/2, q/2]) 2^-16: the Slalom comparator's unmask
-//           and de-quantization (Sec. 6.2); acc and c are exact integers in binary64.
-enum { kOut64 = 0, kUnmask = 1, kSlalom = 2 };
-constexpr double kSlalomQ = 10485767.0;  // 2^23 + 2^21 + 7
-
-__device__ __forceinline__ void finish(double* out64, float* out32, int64_t o, double acc, const double* c, int mode) {
-  if (mode == kOut64) {
-    out64[o] = acc;
-  } else if (mode == kUnmask) {
-    out32[o] = (float)(acc - c[o]);
-  } else {
-    const double t = acc - c[o];  // exact integer, |t| < 2^53
-    double m = t - kSlalomQ * floor(t / kSlalomQ);
-    if (m < 0.0) m += kSlalomQ;
-    if (m >= kSlalomQ) m -= kSlalomQ;
-    if (m > (kSlalomQ - 1.0) * 0.5) m -= kSlalomQ;
-    out32[o] = (float)(m * 0x1p-16);
-  }
-}
-
-// part[split][m][n] (splits > 1) or, with one split, the final value (see finish).
+// part[split][m][n] (splits > 1) or, with one split, the final value (see finish_f64).
 template <typename TA, int MT>
 __global__ void __launch_bounds__(THREADS) gemv_f64_kernel(double* __restrict__ out64, float* __restrict__ out32,
                                                            const TA* __restrict__ A, const float* __restrict__ W,
@@ -134,7 +116,7 @@ __global__ void __launch_bounds__(THREADS) gemv_f64_kernel(double* __restrict__ 
       if (splits > 1)
         out64[(int64_t)split * M * N + o] = acc[r][m];
       else
-        finish(out64, out32, o, acc[r][m], c, mode);
+        finish_f64(out64, out32, o, acc[r][m], c, mode);
     }
   }
 }
@@ -149,7 +131,7 @@ __global__ void __launch_bounds__(256) reduce_f64_kernel(double* __restrict__ ou
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
     double s = part[i];
     for (int sp = 1; sp < splits; ++sp) s += part[(int64_t)sp * total + i];
-    finish(out64, out32, i, s, c, mode);
+    finish_f64(out64, out32, i, s, c, mode);
   }
 }
 
@@ -204,6 +186,12 @@ spl_status run_f64(double* out64, float* out32, const TA* A, const float* W, con
       (out32 && !aligned16(out32)))
     return SPL_EALIGN;
   if (M > 0x7fffffffLL || N > 0x7fffffffLL || K > 0x7fffffffLL) return SPL_ESHAPE;
+  const size_t tc = f64_tc_bytes(M, K, N);
+  if (tc > 0) {
+    if (!ws || ws_bytes < kCounterBytes + tc) return SPL_EWORKSPACE;
+    if (!aligned16(ws)) return SPL_EALIGN;
+    return run_f64_tc(out64, out32, A, W, c, M, K, N, ws, stream, mode);
+  }
   const PlanF64 p = plan_f64(M, K, N);
   if (p.ws > 0 && (!ws || ws_bytes < p.ws)) return SPL_EWORKSPACE;
   if (ws && !aligned16(ws)) return SPL_EALIGN;
@@ -222,7 +210,8 @@ using namespace spl;
 
 extern "C" size_t spl_f64_workspace_bytes(int64_t M, int64_t K, int64_t N) {
   if (M <= 0 || K <= 0 || N <= 0) return 0;
-  return plan_f64(M, K, N).ws;
+  const size_t tc = f64_tc_bytes(M, K, N);
+  return tc > 0 ? kCounterBytes + tc : plan_f64(M, K, N).ws;
 }
 
 extern "C" spl_status spl_precompute_noise_product_f64(double* C, const float* Nz, const float* W, int64_t M,

@@ -45,6 +45,8 @@
 #include <cuda_fp16.h>
 
 #include "common.cuh"
+#include "fp64.cuh"
+#include "noise.cuh"  // packed fp32 pairs
 
 namespace spl {
 
@@ -242,15 +244,15 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 // CTAS = 2: the pair's MMA.  COLL: what it does with the A operand in the tensor core's collector buffer --
 // nothing, keep it for the next MMA, or use (and drop) the one the MMA before kept.
 enum Collect { kCollNone = 0, kCollFill = 1, kCollUse = 2 };
-template <class Md, uint32_t IDESC, int CTAS = 1, int COLL = kCollNone>
-__device__ __forceinline__ void mma(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t accumulate,
-                                    uint32_t leader) {
+template <class Md, int CTAS = 1, int COLL = kCollNone>
+__device__ __forceinline__ void mma_of(uint32_t idesc, uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi,
+                                       uint32_t accumulate, uint32_t leader) {
   static_assert(CTAS == 1 ? COLL == kCollNone : Md::kF16, "pairs and the collector: fp16 pairs only");
 #define SPL_MMA(GROUP_KIND)                                                                                      \
   asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %6, 0;\n\t" \
                "mov.b64 da, {%1, %5};\n\tmov.b64 db, {%2, %5};\n\t"                                              \
                "@q tcgen05.mma.cta_group::" GROUP_KIND " [%0], da, db, %3, p;\n\t}" ::"r"(d_tmem),                \
-               "r"(a_lo), "r"(b_lo), "r"(IDESC), "r"(accumulate), "r"(hi), "r"(leader)                             \
+               "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(accumulate), "r"(hi), "r"(leader)                             \
                : "memory")
   if constexpr (CTAS == 2 && COLL == kCollFill) {
     SPL_MMA("2.kind::f16.collector::a::fill");
@@ -264,6 +266,11 @@ __device__ __forceinline__ void mma(uint32_t d_tmem, uint32_t a_lo, uint32_t b_l
     SPL_MMA("1.kind::tf32");
   }
 #undef SPL_MMA
+}
+template <class Md, uint32_t IDESC, int CTAS = 1, int COLL = kCollNone>
+__device__ __forceinline__ void mma(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t accumulate,
+                                    uint32_t leader) {
+  mma_of<Md, CTAS, COLL>(IDESC, d_tmem, a_lo, b_lo, hi, accumulate, leader);
 }
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
@@ -1402,6 +1409,7 @@ tc_swap_kernel(const __grid_constant__ TcMaps maps, float* __restrict__ out, con
 }
 
 #include "gemm_pair.cuh"
+#include "gemm_f64.cuh"
 
 // ---- host side: tensor maps ------------------------------------------------------
 using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -2129,6 +2137,34 @@ spl_status run_tc_matched(const LinearArgs& a, int64_t order_rows) {
   return run_tc_impl(a, -1, -1, 0, splits);
 }
 
+}  // namespace spl
+
+namespace spl {
+size_t f64_tc_bytes(int64_t M, int64_t K, int64_t N) { return plan_f64_tc(M, K, N).bytes; }
+
+namespace {
+template <class TX>
+spl_status run_f64_tc_impl(double* out64, float* out32, const TX* A, const float* W, const double* c, int64_t M,
+                           int64_t K, int64_t N, void* ws, cudaStream_t stream, int mode) {
+  const F64TcPlan p = plan_f64_tc(M, K, N);
+  char* base = static_cast<char*>(ws) + kCounterBytes;
+  switch (p.tn) {
+    case 16: return launch_f64_tc<16, TX>(p, out64, out32, A, W, c, M, K, N, base, stream, mode);
+    case 32: return launch_f64_tc<32, TX>(p, out64, out32, A, W, c, M, K, N, base, stream, mode);
+    case 64: return launch_f64_tc<64, TX>(p, out64, out32, A, W, c, M, K, N, base, stream, mode);
+  }
+  return SPL_EUNSUPPORTED;
+}
+}  // namespace
+
+spl_status run_f64_tc(double* out64, float* out32, const float* A, const float* W, const double* c, int64_t M,
+                      int64_t K, int64_t N, void* ws, cudaStream_t stream, int mode) {
+  return run_f64_tc_impl<float>(out64, out32, A, W, c, M, K, N, ws, stream, mode);
+}
+spl_status run_f64_tc(double* out64, float* out32, const double* A, const float* W, const double* c, int64_t M,
+                      int64_t K, int64_t N, void* ws, cudaStream_t stream, int mode) {
+  return run_f64_tc_impl<double>(out64, out32, A, W, c, M, K, N, ws, stream, mode);
+}
 }  // namespace spl
 
 // Failure-detection test hook: one TF32X3 product in which the copy of the first K stage is

@@ -1,0 +1,135 @@
+"""The binary64 products as exact slices on the tensor cores, against exact rational sums of the same terms:
+inside gamma_K S (the bound of a binary64 sum in any order, which the header promises) at every edge of the
+tiles, and on the inputs that fixed point alone would get wrong."""
+
+import math
+from fractions import Fraction
+
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+U64 = 2.0 ** -53
+
+
+@pytest.fixture(scope="module")
+def spl():
+    from paper_2609_15039_gb300 import spl as s
+    return s
+
+
+def _product(spl, X, W):
+    """X W^T through the correction (fp32 X) or through the unmask with C = 0, whose result is rounded to fp32."""
+    M, K = X.shape
+    N = W.shape[0]
+    ws = spl.workspace(spl.spl_f64_workspace_bytes(M, K, N))
+    # the slices' workspace: 12 bytes an output and K range, 8 a row
+    assert ws.numel() >= 64 * 1024 + 12 * M * N + 8 * (M + N)
+    if X.dtype == torch.float32:
+        out = torch.full((M, N), float("nan"), device="cuda", dtype=torch.float64)
+        spl.spl_precompute_noise_product_f64(out, X, W, workspace=ws)
+    else:
+        out = torch.full((M, N), float("nan"), device="cuda")
+        spl.spl_masked_linear_unmask_f64(out, X, W, torch.zeros((M, N), device="cuda", dtype=torch.float64),
+                                         workspace=ws)
+    assert spl.spl_get_device_status() == 0
+    return out
+
+
+def _check(spl, X, W, samples):
+    X, W = X.cuda(), W.cuda()
+    got = _product(spl, X, W).double().cpu().numpy()
+    assert np.isfinite(got).all()
+    K = X.shape[1]
+    for m, n in samples:
+        terms = [Fraction(a) * Fraction(b) for a, b in zip(X[m].tolist(), W[n].tolist())]
+        exact, S = sum(terms), float(sum(abs(t) for t in terms))
+        tol = K * U64 / (1 - K * U64) * S + 4 * U64 * abs(float(exact))
+        if X.dtype == torch.float64:
+            tol += 2.0 ** -24 * abs(float(exact)) + 2.0 ** -150  # the result is fp32
+        assert abs(float(Fraction(float(got[m, n])) - exact)) <= tol, (m, n, got[m, n], float(exact), tol)
+
+
+def _sample(M, N, count=24):
+    rng = np.random.default_rng(5)
+    corners = [(0, 0), (M - 1, N - 1), (0, N - 1), (M - 1, 0)]
+    return corners + [(int(rng.integers(M)), int(rng.integers(N))) for _ in range(count)]
+
+
+# tokens at the tile widths and past them, weight rows at 128, K at a chunk, past one, over several K ranges
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("M,K,N", [(1, 8192, 1040), (16, 1024, 300), (17, 1152, 257), (32, 132 * 8, 129), (33, 4100, 128),
+                                   (64, 640, 127), (65, 2052, 513), (130, 4096, 130), (256, 132, 129)])
+def test_slices_match_exact_sums(spl, dtype, M, K, N):
+    g = torch.Generator().manual_seed(M + K + N)
+    X = torch.randn((M, K), generator=g, dtype=torch.float64) * 2.6e8
+    W = torch.randn((N, K), generator=g) * 0.02
+    _check(spl, X.to(dtype), W, _sample(M, N))
+
+
+def test_slices_hold_the_largest_digit_sums(spl):
+    """Every digit at its largest magnitude and of one sign: the accumulators reach their bound, and the sums
+    are exact (53 bits hold them)."""
+    M, K, N = 40, 4096, 256
+    x = -float(0x40808080808080) * 2.0 ** -30
+    w = -float(0x408080) * 2.0 ** -40
+    got = _product(spl, torch.full((M, K), x, dtype=torch.float64, device="cuda"),
+                   torch.full((N, K), w, device="cuda"))
+    exact = float(Fraction(x) * Fraction(w) * K)
+    assert torch.equal(got, torch.full_like(got, exact))
+
+
+def test_slices_of_rows_that_fixed_point_loses(spl):
+    """Large entries that meet zero weights, entries over 120 binades, rows of zeros, denormals: summed again in
+    binary64 where the slices cannot hold the bound."""
+    M, K, N = 24, 1024, 192
+    g = torch.Generator().manual_seed(9)
+    X = torch.randn((M, K), generator=g, dtype=torch.float64)
+    W = torch.randn((N, K), generator=g) * 0.02
+    X[:, 5] = 1e250
+    W[:, 5] = 0.0
+    X[3] = 0.0
+    W[7] = 0.0
+    X[4] = X[4].abs() * 5e-324 * 1000
+    W[9, 1:] = 0.0
+    X[6] = torch.ldexp(torch.randn(K, generator=g, dtype=torch.float64), torch.randint(-60, 60, (K,), generator=g))
+    X[6, 5] = 1.0
+    _check(spl, X, W, [(m, n) for m in (0, 3, 4, 23) for n in (0, 7, 9, 191)])
+    got = _product(spl, X.cuda(), W.cuda())
+    assert torch.equal(got[3], torch.zeros_like(got[3])) and torch.equal(got[:, 7], torch.zeros_like(got[:, 7]))
+
+
+def test_slices_pass_infinities_and_nans_on(spl):
+    M, K, N = 44, 512, 200
+    g = torch.Generator().manual_seed(11)
+    X = torch.randn((M, K), generator=g, dtype=torch.float64).cuda()
+    W = (torch.randn((N, K), generator=g) * 0.02).cuda()
+    clean = _product(spl, X, W)
+    X2, W2 = X.clone(), W.clone()
+    X2[2, 7], X2[5, 9] = float("inf"), float("nan")
+    W2[11, 100], W2[60, 7] = float("nan"), 0.0
+    got = _product(spl, X2, W2)
+    ref = (X2 @ W2.double().T).float()
+    assert torch.equal(torch.isnan(got), torch.isnan(ref)) and torch.equal(torch.isinf(got), torch.isinf(ref))
+    assert torch.equal(got[torch.isinf(ref)], ref[torch.isinf(ref)])
+    keep = torch.ones((M, N), dtype=torch.bool, device="cuda")
+    keep[2], keep[5], keep[:, 11], keep[:, 60] = False, False, False, False
+    assert torch.equal(got[keep], clean[keep])
+
+
+@pytest.mark.parametrize("seed", [1, 2])
+def test_slices_are_closer_than_a_binary64_sum(spl, seed):
+    """No less precise than the FP64 pipe: over noise-like rows of the Down shape the error of the slices, in units
+    of the result's standard deviation, stays below 2^-53 (a binary64 sum of 8192 terms is at 1.8e-16 there)."""
+    M, K, N = 64, 8192, 256
+    g = torch.Generator().manual_seed(seed)
+    X = (torch.randn((M, K), generator=g) * 2.6e8).cuda()
+    W = (torch.randn((N, K), generator=g) * 0.02).cuda()
+    got = _product(spl, X, W)
+    err = []
+    for m, n in _sample(M, N, 60):
+        exact = sum(Fraction(a) * Fraction(b) for a, b in zip(X[m].tolist(), W[n].tolist()))
+        err.append(float(Fraction(float(got[m, n])) - exact))
+    assert math.sqrt(np.mean(np.square(err))) <= U64 * 2.6e8 * 0.02 * math.sqrt(K)
