@@ -4,7 +4,6 @@
 #include <cstdint>
 #include <cmath>
 
-#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include "spl.h"
@@ -18,11 +17,6 @@ constexpr int kNumSMsGB300 = 152;
 // reads it and clears it (synchronously).
 constexpr unsigned int kStatusTimeout = 1u;
 cudaError_t read_clear_device_status(unsigned int* word);
-unsigned int* device_status_word();  // its device address on the current device (null: the lookup failed)
-
-// 2-D tensor map over a row-major [rows, K] matrix of fp32 or fp16 with a box_k x box_rows box.
-bool make_map(CUtensorMap* map, const void* base, bool f16, int64_t rows, int64_t K, int box_k, int box_rows,
-              CUtensorMapSwizzle swz);
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
