@@ -532,7 +532,7 @@ spl_status spl_test_tc_capacity(int64_t tile_n, int64_t ring_kb, int64_t cluster
  * equals the unsplit product bit for bit); it needs splits 1, seg_splits 0,
  * full_tiles 0, a one-CTA-per-SM variant and N % 4 == 0.  ring_kb 448 with
  * tile_n 256, 224, 192, 160 or 128 is the pair kernel (FP16X3, persistent != 0,
- * splits 1, full_tiles 0, N % 4 == 0, any seg_splits whose K ranges are single
+ * splits 1, full_tiles 0, any N and any seg_splits whose K ranges are single
  * accumulation chains: EINVAL otherwise); its results equal the unsplit product's, or
  * the seg_splits-way split's, bit for bit.  path is
  * SPL_PATH_TF32X3 or SPL_PATH_FP16X3.  Same operands, workspace and errors as

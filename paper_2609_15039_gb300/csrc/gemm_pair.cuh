@@ -21,7 +21,8 @@
 // the same order as tc_gemm_kernel's unsplit segmented form, so the result equals it bit for bit.  An
 // accumulator is handed back as soon as it is read, so folding, C and the stores overlap the MMAs of the
 // next segments.  C comes in and the result goes out by TMA, 32 rows x 32 columns per warp at a time
-// through 4 KB of shared memory of the warp's own (rows and columns past the tensor are clipped).
+// through 4 KB of shared memory of the warp's own (rows and columns past the tensor are clipped); where
+// an output row is not a whole number of 16-byte units (N % 4 != 0) the warp writes the 4 KB out row by row.
 //
 // Hand-over: every segment of the CTA's tiles, numbered g = 0, 1, ..., uses accumulator g % 2; its sums are
 // complete at completion g / 2 of buf_full[g % 2] (in each CTA, one multicast commit) and the accumulator
@@ -95,8 +96,9 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
 
 template <int BN>
 __global__ void __launch_bounds__(PAIR_THREADS, 1)
-tc_pair_kernel(const __grid_constant__ TcMaps maps, const int* __restrict__ a_exp, const int* __restrict__ w_exp,
-               int64_t M, int64_t K, int64_t N, int tiles, int m_tiles, int chain, int64_t c_rows) {
+tc_pair_kernel(const __grid_constant__ TcMaps maps, float* __restrict__ out, const float* __restrict__ C,
+               const int* __restrict__ a_exp, const int* __restrict__ w_exp, int64_t M, int64_t K, int64_t N, int tiles,
+               int m_tiles, int chain, int64_t c_rows) {
   using L = PairCfg<BN>;
   constexpr int STAGES = L::STAGES, BK = L::BK;
   extern __shared__ uint8_t smem_raw[];
@@ -302,7 +304,8 @@ tc_pair_kernel(const __grid_constant__ TcMaps maps, const int* __restrict__ a_ex
       const int64_t mw = m0 + 32 * q;  // the warp's first row
       const int64_t m = mw + lane;
       const float sr = m < M ? pow2f(-__ldg(a_exp + m)) : 1.0f;
-      const bool rows_in = mw < M, has_c = rows_in && mw < c_rows;
+      const bool tma_epi = (N & 3) == 0;
+      const bool rows_in = mw < M, has_c = tma_epi && rows_in && mw < c_rows;
       // C's chunk c of this warp into the staging rows, once the last result has been copied out of them
       auto fetch_c = [&](int c) {
         if (lane == 0) {
@@ -360,7 +363,7 @@ tc_pair_kernel(const __grid_constant__ TcMaps maps, const int* __restrict__ a_ex
             if (c > 0) fetch_c(c);
             ok = ok && __all_sync(0xffffffffu, mbar_wait(my_cbar, c_loads & 1u, kWaitNs, abort_flag));
             ++c_loads;
-          } else {
+          } else if (tma_epi) {
             if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
             __syncwarp();
           }
@@ -377,11 +380,23 @@ tc_pair_kernel(const __grid_constant__ TcMaps maps, const int* __restrict__ a_ex
             }
             *dst = o;
           }
-          fence_proxy_async_smem();  // these writes before the copy that reads them
-          __syncwarp();
-          if (lane == 0) {
-            if (ok) tma_store_2d(&maps.y, stage_addr, (int)nc0, (int)mw);
-            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+          if (tma_epi) {
+            fence_proxy_async_smem();  // these writes before the copy that reads them
+            __syncwarp();
+            if (lane == 0) {
+              if (ok) tma_store_2d(&maps.y, stage_addr, (int)nc0, (int)mw);
+              asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+            }
+          } else {
+            __syncwarp();
+            const int64_t n = nc0 + lane;
+#pragma unroll 8
+            for (int r = 0; r < 32; ++r) {
+              const int64_t mr = mw + r, o = mr * N + n;
+              if (mr >= M || n >= N) continue;
+              const float v = reinterpret_cast<const float*>(stage_out)[32 * r + 4 * ((lane >> 2) ^ (r & 7)) + (lane & 3)];
+              out[o] = mr < c_rows ? __fsub_rn(v, __ldcs(C + o)) : v;
+            }
           }
           __syncwarp();
         }

@@ -1518,9 +1518,11 @@ int swap_width_index(int64_t tokens) {
 // below, in us: a round of co-resident CTAs takes F + b K / s (F: setup, pipeline fill, epilogue and
 // cluster reduction; b: the mainloop per 1000 elements of K on FP16X3; TF32X3 takes two k-blocks where
 // FP16X3 takes one).  Fitted to a sweep of every variant, split, persistent and pair form over the eight
-// Llama and Qwen projections at 61 to 2048 rows on GB300 (64 shapes): the picks are within 0.8% of the
-// best form measured on average, 8% at worst (61 rows by 19456 outputs, where HBM is the bound and the
-// model does not see it); the model before the MMA issue was fixed was 10% off on average.
+// Llama and Qwen projections at 61 to 2048 rows on GB300 (64 shapes).  Streaming the weight bounds the few-row
+// shapes whatever the form, so no form counts for less than 6 us + its bytes at HBM's rate, and of forms that
+// would stay below that the one with fewer splits is taken (shape_rank).  The picks are within 0.4% of the
+// best form measured on average, 4% at worst; without the HBM term 0.8% and 8% (128 x 2560 by 19456:
+// clusters of 2 43.1 us, unsplit 40.3), and before the MMA issue was fixed 10% on average.
 struct Variant {
   int bn, rk, cps;
   double F, b;
@@ -1575,7 +1577,7 @@ int max_active_clusters(int v, int s, int sms) {
 }
 
 // Launch shape: a variant, then either one launch with every tile's K split s ways over a cluster, or
-// whole waves of unsplit tiles followed by the remaining tiles split (so the last wave is not mostly
+// (TF32X3) whole waves of unsplit tiles followed by the remaining tiles split (so the last wave is not mostly
 // idle), or one persistent launch, on single SMs or on SM pairs.  At least 256 of K per CTA; ties go to
 // the earlier variant and to fewer splits.
 struct TcShape {
@@ -1583,7 +1585,7 @@ struct TcShape {
   int64_t full_tiles;  // tiles of the first, unsplit launch (whole waves)
   int64_t rest_tiles;  // tiles of the second launch
   int rest_splits;
-  double cost;              // us
+  double cost;              // us (shape_rank)
   bool persistent = false;  // one launch of tc_persistent_kernel over every tile (unsplit)
   int pair = -1;            // >= 0: width index of tc_pair_kernel, one launch over every tile (unsplit)
 };
@@ -1662,7 +1664,14 @@ double launch_cost(int v, int64_t tiles, int64_t K, int s, int sms, bool f16) {
   return (double)ceil_div(tiles, clusters) * (kVariant[v].F + k_cost(kVariant[v].b, K, f16) / (double)s);
 }
 
+// What forms are compared by: the cost, not below what HBM allows, and a little per split.
+double shape_rank(double cost, int splits, double hbm) { return std::max(cost, hbm) + 0.1 * splits; }
+double hbm_us(int64_t M, int64_t K, int64_t N, bool f16) {  // 4 or 8 bytes a weight and an entry of A, C in, Y out
+  return 6.0 + ((double)(N + M) * (double)K * (f16 ? 4.0 : 8.0) + 8.0 * (double)M * (double)N) / 6.7e6;
+}
+
 TcShape tc_shape_for(int v, int64_t M, int64_t K, int64_t N, int sms, bool f16) {
+  const double hbm = hbm_us(M, K, N, f16);
   // the persistent epilogue stores whole float4s: output rows of whole 16-byte units (a launch whose
   // pointers are not 16-byte aligned runs the same tiles unsplit in tc_gemm_kernel: the same sums)
   const bool persistent_ok = (N & 3) == 0;
@@ -1670,23 +1679,26 @@ TcShape tc_shape_for(int v, int64_t M, int64_t K, int64_t N, int sms, bool f16) 
   const int max_s = (int)std::max<int64_t>(1, std::min<int64_t>(MAX_CLUSTER, K / 256));
   TcShape best{v, 0, tiles, 1, 1e300};
   for (int s = 1; s <= max_s; ++s) {
-    const double c = launch_cost(v, tiles, K, s, sms, f16);
+    const double c = shape_rank(launch_cost(v, tiles, K, s, sms, f16), s, hbm);
     if (c < best.cost * (1.0 - 1e-9)) best = TcShape{v, 0, tiles, s, c};
   }
   const int64_t wave = max_active_clusters(v, 1, sms);
-  // whole waves of unsplit tiles, cut at whole columns of tiles (M is the fast index), so that every
-  // output row of a column is summed the same way wherever it sits in M
+  // TF32X3: whole waves of unsplit tiles, cut at whole columns of tiles (M is the fast index), so that every
+  // output row of a column is summed the same way wherever it sits in M.  FP16X3 leaves such launches to the
+  // pairs: a correction cannot follow two orders at once, so the rounding of a product in two launches does
+  // not cancel in the unmask (264 x 3072 by 16384: 81 us but 2.4 times the error, 85 us in one launch).
   const int64_t m_tiles = ceil_div(M, BM);
   const int64_t full = (tiles / wave) * wave / m_tiles * m_tiles, rest = tiles - full;
-  if (full > 0 && rest > 0) {
+  if (!f16 && full > 0 && rest > 0) {
     const double cf = launch_cost(v, full, K, 1, sms, f16);
     for (int s = 1; s <= max_s; ++s) {
-      const double c = cf + launch_cost(v, rest, K, s, sms, f16);
+      const double c = shape_rank(cf + launch_cost(v, rest, K, s, sms, f16), s, hbm);
       if (c < best.cost * (1.0 - 1e-9)) best = TcShape{v, full, rest, s, c};
     }
   }
   if (persistent_ok && kVariant[v].cps == 1 && tiles > wave) {  // more than one wave of unsplit tiles
-    const double c = kVariant[v].F + (double)ceil_div(tiles, wave) * (k_cost(kVariant[v].b, K, f16) + kPersistentTile);
+    const double c = shape_rank(
+        kVariant[v].F + (double)ceil_div(tiles, wave) * (k_cost(kVariant[v].b, K, f16) + kPersistentTile), 1, hbm);
     if (c < best.cost * (1.0 - 1e-9)) {
       best = TcShape{v, 0, tiles, 1, c};
       best.persistent = true;
@@ -1695,14 +1707,12 @@ TcShape tc_shape_for(int v, int64_t M, int64_t K, int64_t N, int sms, bool f16) 
   return best;
 }
 
-// The cheapest pair form, if it beats `best` (FP16X3, output rows of whole 16-byte units): M and N in tiles
-// of the widths, every one unsplit.  rest_tiles counts 128-row tiles, as the other forms do.
-void consider_pairs(TcShape& best, int64_t M, int64_t K, int64_t N) {
-  if ((N & 3) != 0) return;
+// The cheapest pair form, if it beats `best` (FP16X3): M and N in tiles of the widths, every one unsplit.  rest_tiles counts 128-row tiles, as the other forms do.
+void consider_pairs(TcShape& best, int64_t M, int64_t K, int64_t N, double hbm) {
   for (int w = 0; w < kPairs; ++w) {
     const int64_t cols = ceil_div(N, (int64_t)kPair[w].bn), tiles = ceil_div(M, (int64_t)256) * cols;
-    const double c =
-        kPair[w].F + (double)ceil_div(tiles, (int64_t)pairs_of(w)) * (k_cost(kPair[w].b, K, true) + kPair[w].h);
+    const double c = shape_rank(
+        kPair[w].F + (double)ceil_div(tiles, (int64_t)pairs_of(w)) * (k_cost(kPair[w].b, K, true) + kPair[w].h), 1, hbm);
     if (c < best.cost * (1.0 - 1e-9)) {
       best = TcShape{0, 0, ceil_div(M, BM) * cols, 1, c};
       best.pair = w;
@@ -1735,7 +1745,7 @@ TcShape tc_bank_shape(int64_t M, int64_t K, int64_t N, int seg_splits, int sms, 
   }
   // segments longer than a chain belong to ranks that fold chains of their own: only a split reproduces them
   if (f16 && (seg_splits == 1 || rank_blocks_of<Fp16x3>(K, seg_splits) <= kChainBlocks))
-    consider_pairs(best, M, K, N);
+    consider_pairs(best, M, K, N, 0.0);
   return best;
 }
 
@@ -1745,7 +1755,7 @@ TcShape tc_shape(int64_t M, int64_t K, int64_t N, int sms, bool f16) {
     const TcShape t = tc_shape_for(v, M, K, N, sms, f16);
     if (t.cost < best.cost * (1.0 - 1e-9)) best = t;
   }
-  if (f16) consider_pairs(best, M, K, N);
+  if (f16) consider_pairs(best, M, K, N, hbm_us(M, K, N, f16));
   return best;
 }
 
@@ -1863,7 +1873,8 @@ template <int BN>
 spl_status launch_pair_bn(const LinearArgs& a, const uint16_t* a_hi, const uint16_t* a_lo, const int* a_exp, int chain) {
   using L = PairCfg<BN>;
   if (!set_smem_attr_pair<BN>()) return SPL_ECUDA;
-  if ((a.N & 3) != 0 || !aligned16(a.out) || (a.c && !aligned16(a.c))) return SPL_EALIGN;  // whole 16-byte units
+  const bool tma_epi = (a.N & 3) == 0;  // output rows of whole 16-byte units
+  if (tma_epi && (!aligned16(a.out) || (a.c && !aligned16(a.c)))) return SPL_EALIGN;
   const int64_t m_tiles = ceil_div(a.M, (int64_t)256), tiles = m_tiles * ceil_div(a.N, (int64_t)BN);
   if (tiles > 0x3fffffffLL) return SPL_ESHAPE;
   TcMaps maps;
@@ -1873,8 +1884,8 @@ spl_status launch_pair_bn(const LinearArgs& a, const uint16_t* a_hi, const uint1
       !make_map(&maps.a_lo, a_lo, true, a.M, a.K, L::BK, 128, CU_TENSOR_MAP_SWIZZLE_128B) ||
       !make_map(&maps.w_hi, a.w_h16, true, a.N, a.K, L::BK, BN / 2, CU_TENSOR_MAP_SWIZZLE_128B) ||
       !make_map(&maps.w_lo, a.w_l16, true, a.N, a.K, L::BK, BN / 2, CU_TENSOR_MAP_SWIZZLE_128B) ||
-      !make_map(&maps.y, a.out, false, a.M, a.N, 32, 32, CU_TENSOR_MAP_SWIZZLE_128B) ||
-      (c_rows > 0 && !make_map(&maps.c, a.c, false, c_rows, a.N, 32, 32, CU_TENSOR_MAP_SWIZZLE_128B)))
+      (tma_epi && !make_map(&maps.y, a.out, false, a.M, a.N, 32, 32, CU_TENSOR_MAP_SWIZZLE_128B)) ||
+      (tma_epi && c_rows > 0 && !make_map(&maps.c, a.c, false, c_rows, a.N, 32, 32, CU_TENSOR_MAP_SWIZZLE_128B)))
     return SPL_ECUDA;
   const int64_t pairs = std::min<int64_t>(tiles, active_pairs<BN>());
   cudaLaunchConfig_t cfg;
@@ -1892,8 +1903,8 @@ spl_status launch_pair_bn(const LinearArgs& a, const uint16_t* a_hi, const uint1
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, tc_pair_kernel<BN>, maps, a_exp, (const int*)a.w_exp, a.M, a.K, a.N,
-                                           (int)tiles, (int)m_tiles, chain, c_rows);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, tc_pair_kernel<BN>, maps, a.out, a.c, a_exp, (const int*)a.w_exp,
+                                           a.M, a.K, a.N, (int)tiles, (int)m_tiles, chain, c_rows);
   note_launches(1);
   return e == cudaSuccess ? SPL_OK : SPL_ECUDA;
 }
@@ -2238,7 +2249,7 @@ extern "C" spl_status spl_test_tc_product(float* out, const float* A, const spl_
   if (v < 0 && pair < 0) return SPL_EINVAL;
   if (pair >= 0) {  // every tile unsplit on the pair kernel
     if (path != SPL_PATH_FP16X3 || splits != 1 || full_tiles != 0 || !persistent || seg_splits < 0 ||
-        seg_splits > MAX_CLUSTER || (N & 3) != 0)
+        seg_splits > MAX_CLUSTER)
       return SPL_EINVAL;
     if ((K & 3) != 0) return SPL_EALIGN;
     if (!aligned16(out) || !aligned16(A) || (C && !aligned16(C))) return SPL_EALIGN;

@@ -29,10 +29,11 @@ def _problem(spl, M, K, N, seed):
 
 
 # (rows, K, outputs past a whole tile): one row, the two CTAs' boundary, a ragged second row tile; one k-block,
-# an odd number of them, one element of K past a chain, several chains; a last tile of 4 columns or none
+# an odd number of them, one element of K past a chain, several chains; a last tile of 4 columns or none, output rows
+# that are no whole number of 16-byte units
 @pytest.mark.parametrize("bn", WIDTHS)
 @pytest.mark.parametrize("M,K,extra", [(1, 32, 4), (128, 8, 0), (129, 96, 36), (256, 1024, 0), (257, 1032, 4),
-                                       (300, 3080, 100)])
+                                       (300, 3080, 100), (161, 64, 1), (290, 1096, 35)])
 def test_pair_equals_unsplit_product(spl, bn, M, K, extra):
     N = bn + extra
     W, X, C, ws = _problem(spl, M, K, N, seed=11)
@@ -70,11 +71,12 @@ def test_pair_segments_equal_split_product(spl, K, s):
     assert spl.spl_get_device_status() == 0
 
 
+@pytest.mark.parametrize("N", [16384, 16383])
 @pytest.mark.parametrize("M", [4, 100, 128, 488])
-def test_library_pair_product_with_fewer_correction_rows(spl, M):
+def test_library_pair_product_with_fewer_correction_rows(spl, M, N):
     """The stacked call on the pair kernel: C has M rows, the rows after them are corrections, equal to the
     product without C bit for bit (the boundary inside a warp's 32 rows, at a CTA's and past a tile's end)."""
-    rows, K, N = 1000, 1024, 16384
+    rows, K = 1000, 1024
     assert spl.spl_test_tc_shape(rows, K, N)[1] == PAIR_RING
     W, X, C, ws = _problem(spl, rows, K, N, seed=41)
     plain, YC = torch.empty((rows, N), device="cuda"), torch.full((rows, N), float("nan"), device="cuda")
