@@ -10,8 +10,8 @@
 // them into an FMA, so the eta written to N is exactly the eta added to x.
 //
 // Layout: one thread handles one Philox block (4 consecutive elements) per
-// step as a float4; two blocks are in flight per loop trip.  The grid is a
-// whole number of waves over the SMs (grid-stride loop).
+// step as a float4; two or four blocks are in flight per loop trip.  The grid is a
+// whole number of blocks per SM (grid-stride loop).
 
 #include <algorithm>
 
@@ -26,6 +26,11 @@ namespace {
 constexpr int kThreads = 256;
 
 // xt = x + eta (if xt), nout = eta (if nout).  n elements, nb = ceil(n/4) Philox blocks.
+// What bounds it, at 1e8 entries (800 MB, 120 us at the copy rate): without noise the loads in flight, so four blocks
+// a trip (two: 136 us, four: 120); the Laplace draw the wait for those loads too (149 -> 135 us); the Gaussian
+// draw the instructions (37 an entry, 2.7 to 2.9 issued a cycle of 4, 137 us with nothing read), where two
+// blocks a trip leave more registers (four: 154 us).  16 blocks an SM instead of 8 even out the end of the
+// grid (Gaussian 147 -> 143 us).
 template <int MECH>
 __global__ void __launch_bounds__(kThreads) noise_mask_kernel(float* xt, float* __restrict__ nout,
                                                               const float* x, int64_t n, float b,
@@ -40,22 +45,17 @@ __global__ void __launch_bounds__(kThreads) noise_mask_kernel(float* xt, float* 
   const float4* x4 = reinterpret_cast<const float4*>(x);
   float4* xt4 = reinterpret_cast<float4*>(xt);
   float4* n4 = reinterpret_cast<float4*>(nout);
-  // two blocks per trip: issue both loads first
-  for (; i + stride < nb_full; i += 2 * stride) {
-    float4 xa, xb;
-    if (xt) {
-      xa = __ldcs(x4 + i);
-      xb = __ldcs(x4 + i + stride);
-    }
-    const float4 ea = draw_block<MECH>((uint64_t)i + offset, key, b);
-    const float4 eb = draw_block<MECH>((uint64_t)(i + stride) + offset, key, b);
-    if (nout) {
-      __stcs(n4 + i, ea);
-      __stcs(n4 + i + stride, eb);
-    }
-    if (xt) {
-      __stcs(xt4 + i, add4(xa, ea));
-      __stcs(xt4 + i + stride, add4(xb, eb));
+  constexpr int PER = MECH == kGaussian ? 2 : 4;  // blocks per trip, their loads issued first
+  for (; i + (PER - 1) * stride < nb_full; i += PER * stride) {
+    float4 xv[PER];
+#pragma unroll
+    for (int u = 0; u < PER; ++u)
+      if (xt) xv[u] = __ldcs(x4 + i + u * stride);
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+      const float4 e = draw_block<MECH>((uint64_t)(i + u * stride) + offset, key, b);
+      if (nout) __stcs(n4 + i + u * stride, e);
+      if (xt) __stcs(xt4 + i + u * stride, add4(xv[u], e));
     }
   }
   for (; i < nb_full; i += stride) {
@@ -388,7 +388,7 @@ spl_status launch_noise_mask(float* xt, float* nout, const float* x, int64_t n, 
                              spl_mech mech, spl_rng rng, cudaStream_t stream) {
   if ((reinterpret_cast<uintptr_t>(rng.offset_dev) & 7u) != 0) return SPL_EALIGN;
   const float b = std::isinf(eps) ? 0.0f : (float)(sensitivity / eps);
-  const int grid = grid_for(ceil_div(n, 4), 8);
+  const int grid = grid_for(ceil_div(n, 4), 16);
   const PhiloxKey key = make_philox_key(rng.seed, rng.stream_id);
   if (b == 0.0f) {
     return launch_pdl(noise_mask_kernel<kZero>, dim3(grid), dim3(kThreads), 0, stream, xt, nout, x, n, b, key, rng.offset, rng.offset_dev);

@@ -54,11 +54,6 @@ struct F64Cfg {
 // down r = 256 t + M rounds to the digit (M = 1.5 2^23), d = r - M, t' = 256 t - d: every step but the
 // rounding to d is exact (t' is a multiple of t's last place), so the last remainder, at most half of the
 // last digit's unit, is all that is lost.
-__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
-  unsigned long long d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
 __device__ __forceinline__ uint32_t half_pair(unsigned long long v) {
   float a, b;
   up2(v, a, b);
