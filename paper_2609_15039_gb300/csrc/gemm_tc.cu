@@ -110,7 +110,11 @@ struct Cfg {
   static_assert(RK == 96 || RK == 192 || RK == 224, "ring size");
   static constexpr uint32_t A_HALF = BM * Md::BK * Md::ESZ, B_HALF = BN * Md::BK * Md::ESZ;
   static constexpr uint32_t A_HI = 0, A_LO = A_HALF, W_HI = 2 * A_HALF, W_LO = W_HI + B_HALF;
-  static constexpr uint32_t STAGE = W_LO + B_HALF;  // bytes TMA brings per stage
+  static constexpr uint32_t STAGE = W_LO + B_HALF;
+  // Bytes TMA brings per stage when its copies of A have a_rows rows.
+  static __device__ __forceinline__ uint32_t stage_tx(int a_rows) {
+    return 2 * B_HALF + 2u * (uint32_t)(a_rows * Md::BK * Md::ESZ);
+  }
   static constexpr uint32_t RING = RK * 1024;
   static constexpr int STAGES = (int)(RING / STAGE);
   static constexpr int CTAS_PER_SM = RK == 96 ? 2 : 1;
@@ -355,6 +359,12 @@ __device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
   return v;
 }
 
+// Rows of the copies of A: a whole tile, or, when A has fewer rows than one, those it has.  The tile's other rows
+// in shared memory then keep whatever they held, and so do their accumulator rows, which nothing stores.  Zeros
+// for rows that are not there cost as much as copies: with boxes of 128 rows 24 rows by 2560 by 19456 took 50 to
+// 62 us (36 with boxes of 24) and 61 rows 37.8 (36.9).
+__host__ __device__ __forceinline__ int a_box_rows(int64_t M) { return M >= BM ? BM : (int)((M + 7) & ~int64_t(7)); }
+
 struct TcMaps {
   CUtensorMap a_hi, a_lo, w_hi, w_lo;
   CUtensorMap y, c;  // TMA epilogue: the output and C as [M, N] fp32, 32 x 128 boxes, 128-byte swizzle
@@ -500,13 +510,14 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, float* __restrict__ out, con
     uint32_t issued_mask = 0u, phase_mask = 0u;  // per stage: a load was issued / its parity
     bool ok = true;
     const uint64_t pol_w = l2_evict_first(), pol_a = l2_evict_last();
+    const uint32_t stage_tx = L::stage_tx(a_box_rows(M));
     const int pre = nk < STAGES ? nk : STAGES;
     for (int kb = 0; kb < pre; ++kb) {  // fresh ring: every stage is free
       if (kb == skip_kblock) continue;  // failure-detection test only: this stage never arrives
       if (lane == 0) {
         const uint32_t st = smem_u32(smem + (size_t)kb * L::STAGE);
         const int kx = (int)(kbeg + (int64_t)kb * BK);
-        mbar_expect_tx(full_bar(kb), L::STAGE);
+        mbar_expect_tx(full_bar(kb), stage_tx);
         tma_load_2d(st + L::W_HI, &maps.w_hi, full_bar(kb), kx, (int)n0, pol_w);
         tma_load_2d(st + L::W_LO, &maps.w_lo, full_bar(kb), kx, (int)n0, pol_w);
       }
@@ -532,7 +543,7 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, float* __restrict__ out, con
       if (lane == 0) {
         const uint32_t st = smem_u32(smem + (size_t)s * L::STAGE);
         const int kx = (int)(kbeg + (int64_t)kb * BK);
-        mbar_expect_tx(full_bar(s), L::STAGE);
+        mbar_expect_tx(full_bar(s), stage_tx);
         tma_load_2d(st + L::A_HI, &maps.a_hi, full_bar(s), kx, (int)m0, pol_a);
         tma_load_2d(st + L::A_LO, &maps.a_lo, full_bar(s), kx, (int)m0, pol_a);
         tma_load_2d(st + L::W_HI, &maps.w_hi, full_bar(s), kx, (int)n0, pol_w);
@@ -845,6 +856,7 @@ tc_persistent_kernel(const __grid_constant__ TcMaps maps, float* __restrict__ ou
     uint32_t issued_mask = 0u, phase_mask = 0u;
     bool ok = true;
     const uint64_t pol_w = l2_evict_first(), pol_a = l2_evict_last();
+    const uint32_t stage_tx = L::stage_tx(a_box_rows(M));
     pdl_wait();  // A comes from the kernel before this one
     uint32_t it = 0;
     for (int i = 0; i < my_tiles && ok; ++i) {
@@ -860,7 +872,7 @@ tc_persistent_kernel(const __grid_constant__ TcMaps maps, float* __restrict__ ou
         if (lane == 0) {
           const uint32_t sa = smem_u32(smem + (size_t)st * L::STAGE);
           const int kx = kb * BK;
-          mbar_expect_tx(full_bar(st), L::STAGE);
+          mbar_expect_tx(full_bar(st), stage_tx);
           tma_load_2d(sa + L::A_HI, &maps.a_hi, full_bar(st), kx, (int)m0, pol_a);
           tma_load_2d(sa + L::A_LO, &maps.a_lo, full_bar(st), kx, (int)m0, pol_a);
           tma_load_2d(sa + L::W_HI, &maps.w_hi, full_bar(st), kx, (int)n0, pol_w);
@@ -1794,8 +1806,8 @@ spl_status launch_tc(const LinearArgs& a, const uint16_t* a_hi, const uint16_t* 
   const bool f16 = Md::kF16;
   const void* whi = f16 ? (const void*)a.w_h16 : (const void*)a.w_hi;
   const void* wlo = f16 ? (const void*)a.w_l16 : (const void*)a.w_lo;
-  if (!make_map(&maps.a_hi, a_hi, f16, a.M, a.K, Md::BK, BM, CU_TENSOR_MAP_SWIZZLE_64B) ||
-      !make_map(&maps.a_lo, a_lo, f16, a.M, a.K, Md::BK, BM, CU_TENSOR_MAP_SWIZZLE_64B) ||
+  if (!make_map(&maps.a_hi, a_hi, f16, a.M, a.K, Md::BK, a_box_rows(a.M), CU_TENSOR_MAP_SWIZZLE_64B) ||
+      !make_map(&maps.a_lo, a_lo, f16, a.M, a.K, Md::BK, a_box_rows(a.M), CU_TENSOR_MAP_SWIZZLE_64B) ||
       !make_map(&maps.w_hi, whi, f16, a.N, a.K, Md::BK, BN, CU_TENSOR_MAP_SWIZZLE_64B) ||
       !make_map(&maps.w_lo, wlo, f16, a.N, a.K, Md::BK, BN, CU_TENSOR_MAP_SWIZZLE_64B))
     return SPL_ECUDA;
