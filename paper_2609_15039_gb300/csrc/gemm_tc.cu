@@ -39,6 +39,7 @@
 // returns.  Role loops run warp-wide (lane 0 issues), so no warp is diverged at a barrier.
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 
 #include <cuda.h>
@@ -1945,18 +1946,34 @@ spl_status launch_variant(const LinearArgs& a, const uint16_t* hi, const uint16_
   }
 }
 
-// CTAs per token tile of the swapped kernel.  Measured on GB300 (the eight Llama and Qwen
-// projections at 8 and 16 rows): runs of whole tiles are fastest where the weight tiles number
-// between 3/4 of the SMs and all of them (one tile per CTA, no partial tiles: Qwen Gate|Up, 152
-// tiles); otherwise 3/4 of the SMs beat all of them by 0.3-1.5 us, fewer partial tiles to sum
-// outweighing the longer runs, and 1/2 of them lost 1-4 us.  More tiles than SMs: one CTA per SM.
+// CTAs per token tile of the swapped kernel: a whole number k of CTAs for every weight tile, so that no run crosses
+// a tile's end (a run that does sums two pieces, and both tiles wait for it), with k from a model in us: streaming
+// at what one CTA takes (0.37 us for a block of 64 of K) or HBM gives all of them, whichever is slower, and the
+// meeting of the k pieces.  Measured at 16 rows against 3/4 of the SMs whatever the tiles: 3072 by 5120 17.4
+// against 18.4 us (k = 3), 2560 by 6144 17.2 against 18.1 (3), 2048 by 8192 17.4 against 19.3 (2), 4096 by 11008
+// 32.9 against 39.2 (1), 1024 by 4096 9.7 against 11.4 (4).
+// Longer pieces would serve short K better still (256 by 512 with k = 1: 5.1 against 7.9 us), but a longer chain
+// of MMAs rounds more (error 1.3 times as large there), so chains stay as short as 3/4 of the SMs make them; where
+// no k does that, and with more tiles than SMs, the runs are those of 3/4 or all of the SMs.
 int swap_ctas(int64_t K, int64_t N, int sms) {
-  const int64_t w_tiles = ceil_div(N, BM);
-  const int64_t total = w_tiles * ceil_div(K, (int64_t)SwapCfg<16>::BK);
-  int64_t c = 3 * (int64_t)sms / 4;
-  if (w_tiles > sms) c = sms;
-  else if (4 * w_tiles >= 3 * (int64_t)sms) c = w_tiles;
-  return (int)std::max<int64_t>(1, std::min<int64_t>(c, total));
+  const int64_t w_tiles = ceil_div(N, BM), nkb = ceil_div(K, (int64_t)SwapCfg<16>::BK), total = w_tiles * nkb;
+  const int64_t even = w_tiles > sms ? sms : std::max<int64_t>(1, std::min<int64_t>(3 * (int64_t)sms / 4, total));
+  constexpr int64_t chain = 1024 / SwapCfg<16>::BK;
+  const int64_t longest = std::min(chain, 4 * w_tiles >= 3 * (int64_t)sms ? nkb : ceil_div(total, even));
+  const double hbm = (double)total * 32768.0 / 6.7e6;
+  int64_t best_c = even;
+  double best = 1e300;
+  for (int64_t k = 1; k * w_tiles <= sms && k <= nkb; ++k) {
+    const int64_t piece = ceil_div(nkb, k);
+    if (std::min(chain, piece) > longest) continue;
+    const double stream = 0.37 * (double)piece;
+    const double c = std::pow(std::pow(stream, 4.0) + std::pow(hbm, 4.0), 0.25) + (k > 1 ? 2.4 + 0.15 * (double)k : 0.0);
+    if (c < best * (1.0 - 1e-9)) {
+      best = c;
+      best_c = k * w_tiles;
+    }
+  }
+  return (int)best_c;
 }
 
 // Workspace of the swapped kernel's partial tiles: two slots per CTA and token tile of width tn.

@@ -1,5 +1,5 @@
 """Products with fewer rows than the 128 of a tile: the tensor-core kernels copy only the rows there are, the
-tile's other rows keep what shared memory held."""
+tile's other rows keep what shared memory held; and the swapped kernel's split of 9 to 16 rows."""
 
 import pytest
 import torch
@@ -40,4 +40,27 @@ def test_rows_that_are_not_there_do_not_matter(spl, M, path, tile_n, ring_kb, sp
     assert torch.equal(Y, full[:M])
     spl.spl_test_tc_product(Y, X[:M], W, None, **kw)
     assert_product_close(f32(Y), f32(X[:M]), f32(W.w), path, what=f"{M} rows")
+    assert spl.spl_get_device_status() == 0
+
+
+# one tile; pieces of one k-block; several whole pieces a tile; a short last tile and k-block; one tile a CTA; more
+# tiles than SMs; a width where no whole number of CTAs keeps the chains short
+@pytest.mark.parametrize("K,N", [(8, 4), (256, 512), (1024, 1024), (2560, 6144), (1000, 2500), (256, 19456),
+                                 (128, 20000), (512, 11008)])
+@pytest.mark.parametrize("M", [9, 16])
+def test_swapped_split_matches_bank(spl, M, K, N):
+    """The library's product of 9 and 16 rows, and the same noise rows in a bank of 5 draws, whose sums must agree
+    bit for bit."""
+    W = spl.Weight.prepare(wl.weight(N, K, seed=7, device="cuda"), tf32=False)
+    X = wl.activations(5 * M, K, seed=8, device="cuda")
+    ws = spl.workspace(max(spl.spl_linear_workspace_bytes(M, K, N, "fp16x3"),
+                           spl.spl_precompute_matched_workspace_bytes(5 * M, K, N, M, "fp16x3")))
+    bank, Y = torch.empty((5 * M, N), device="cuda"), torch.full((M, N), float("nan"), device="cuda")
+    spl.spl_precompute_noise_product_matched(bank, X, W, M, path="fp16x3", workspace=ws)
+    zero = torch.zeros((M, N), device="cuda")
+    for d in (0, 4):
+        rows = X[d * M:(d + 1) * M].contiguous()
+        spl.spl_masked_linear_unmask(Y, rows, W, zero, path="fp16x3", workspace=ws)
+        assert torch.equal(Y, bank[d * M:(d + 1) * M])
+        assert_product_close(f32(Y), f32(rows), f32(W.w), "fp16x3", what=f"{K} by {N}")
     assert spl.spl_get_device_status() == 0
