@@ -316,6 +316,8 @@ tc_pair_kernel(const __grid_constant__ TcMaps maps, float* __restrict__ out, con
         __syncwarp();
       };
       if (has_c && nc > 0 && n0 + 32 * c_lo < N) fetch_c(0);  // in flight during the tile's mainloop
+      if (!tma_epi && m < c_rows)  // the warp's rows of C into L2 meanwhile
+        for (int64_t n = n0 + 32 * c_lo; n < n0 + 32 * (c_lo + nc) && n < N; n += 32) prefetch_l2(C + m * N + n);
       float run[L::G0][32];
       // segment g's sums are complete: its accumulator (false: gave up)
       auto take = [&](uint32_t& base) {
@@ -388,14 +390,20 @@ tc_pair_kernel(const __grid_constant__ TcMaps maps, float* __restrict__ out, con
               asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             }
           } else {
+            // output rows of no whole 16-byte units: lanes along a row, all 32 rows of C in flight at once
+            // (one row after the other: 469 us at 952 by 80 by 26301, 143 so)
+            const bool col = nc0 + lane < N;
+            const int64_t o0 = mw * N + nc0 + lane;
+            const int live = col ? (int)std::min<int64_t>(32, M - mw) : 0;
+            const int c_end = col && mw < c_rows ? (int)std::min<int64_t>(32, c_rows - mw) : 0;
+            float cc[32];
+#pragma unroll
+            for (int r = 0; r < 32; ++r) cc[r] = r < c_end ? __ldcs(C + o0 + r * N) : 0.f;
             __syncwarp();
-            const int64_t n = nc0 + lane;
-#pragma unroll 8
+#pragma unroll
             for (int r = 0; r < 32; ++r) {
-              const int64_t mr = mw + r, o = mr * N + n;
-              if (mr >= M || n >= N) continue;
               const float v = reinterpret_cast<const float*>(stage_out)[32 * r + 4 * ((lane >> 2) ^ (r & 7)) + (lane & 3)];
-              out[o] = mr < c_rows ? __fsub_rn(v, __ldcs(C + o)) : v;
+              if (r < live) out[o0 + r * N] = r < c_end ? __fsub_rn(v, cc[r]) : v;
             }
           }
           __syncwarp();

@@ -372,16 +372,16 @@ struct TcMaps {
 };
 
 // Rows r0..r1 of the staged tile: the S partial tiles of the cluster summed in rank order (S = 1:
-// this CTA's own), minus C, stored.  A thread takes P float4 positions per batch and issues every
-// load of the batch -- S partials and C for each -- before it adds anything, about 16 loads in
-// flight per thread whatever S is, so the epilogue streams instead of waiting load by load.
+// this CTA's own), minus C, stored; or, with `ragged`, left in this CTA's staged tile, whose rows r0..r1 no other
+// CTA reads.  A thread takes P float4 positions per batch and issues every load of the batch -- S partials and C
+// for each -- before it adds anything, about 16 loads in flight per thread whatever S is, so the epilogue streams
+// instead of waiting load by load.
 template <int S, int BN>
-__device__ __forceinline__ void reduce_store(const float* red, int r0, int r1, int64_t m0, int64_t n0, int64_t M,
+__device__ __forceinline__ void reduce_store(float* red, bool ragged, int r0, int r1, int64_t m0, int64_t n0, int64_t M,
                                              int64_t N, const float* __restrict__ C, float* __restrict__ out,
                                              int64_t c_rows) {
   constexpr int RS = BN + 4;
   constexpr int P = S >= 8 ? 2 : (S >= 4 ? 4 : 8);
-  const bool vec = (N & 3) == 0;
   const uint32_t red_base = smem_u32(red);
   const int total = (r1 - r0) * (BN / 4);
   for (int base = threadIdx.x; base < total; base += THREADS * P) {
@@ -402,7 +402,7 @@ __device__ __forceinline__ void reduce_store(const float* red, int r0, int r1, i
 #pragma unroll
         for (int q = 0; q < S; ++q) part[u][q] = ld_cluster_f4(map_to_rank(off, (uint32_t)q));
       }
-      if (C && m < c_rows && vec && n + 4 <= N) cc[u] = __ldcs(reinterpret_cast<const float4*>(C + m * N + n));
+      if (C && !ragged && m < c_rows) cc[u] = __ldcs(reinterpret_cast<const float4*>(C + m * N + n));
     }
 #pragma unroll
     for (int u = 0; u < P; ++u) {
@@ -415,19 +415,44 @@ __device__ __forceinline__ void reduce_store(const float* red, int r0, int r1, i
       for (int q = 1; q < S; ++q)  // summed in rank order
         v = make_float4(__fadd_rn(v.x, part[u][q].x), __fadd_rn(v.y, part[u][q].y), __fadd_rn(v.z, part[u][q].z),
                         __fadd_rn(v.w, part[u][q].w));
-      float* o = out + m * N + n;
-      const bool has_c = C && m < c_rows;
-      if (vec && n + 4 <= N) {
-        if (has_c)
-          v = make_float4(__fsub_rn(v.x, cc[u].x), __fsub_rn(v.y, cc[u].y), __fsub_rn(v.z, cc[u].z),
-                          __fsub_rn(v.w, cc[u].w));
-        *reinterpret_cast<float4*>(o) = v;
-      } else {
-        const float vv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (n + j < N) o[j] = has_c ? __fsub_rn(vv[j], C[m * N + n + j]) : vv[j];
+      if (ragged) {
+        *reinterpret_cast<float4*>(red + r * RS + c) = v;
+        continue;
       }
+      if (C && m < c_rows)
+        v = make_float4(__fsub_rn(v.x, cc[u].x), __fsub_rn(v.y, cc[u].y), __fsub_rn(v.z, cc[u].z),
+                        __fsub_rn(v.w, cc[u].w));
+      *reinterpret_cast<float4*>(out + m * N + n) = v;
+    }
+  }
+}
+
+// Rows r0..r1 of the staged sums minus C, stored, where the output's rows are no whole 16-byte units (N % 4 != 0):
+// by single elements, a warp's lanes along a row, so that C and the output move in whole lines, and P elements of C
+// in flight per thread.  (Four neighbours a thread, each C loaded where it was subtracted, took 24.1 us for 128 rows
+// of 3072 by 5121 where this takes 22.4, and 22.9 for 61 of 2560 by 6143 where this takes 21.2.)
+template <int BN>
+__device__ __forceinline__ void store_ragged(const float* red, int r0, int r1, int64_t m0, int64_t n0, int64_t M,
+                                             int64_t N, const float* __restrict__ C, float* __restrict__ out,
+                                             int64_t c_rows) {
+  constexpr int RS = BN + 4, P = 32;
+  const int cols = (int)std::min<int64_t>(BN, N - n0);
+  const int rows = (int)std::min<int64_t>(r1, M - m0) - r0;
+  const int c_end = C && m0 < c_rows ? (int)std::min<int64_t>(r1, c_rows - m0) - r0 : 0;  // rows below it subtract C
+  const int64_t origin = (m0 + r0) * N + n0;
+  for (int base = threadIdx.x; base < rows * BN; base += THREADS * P) {
+    float cc[P];
+#pragma unroll
+    for (int u = 0; u < P; ++u) {
+      const int r = (base + u * THREADS) / BN, c = (base + u * THREADS) % BN;
+      cc[u] = c < cols && r < rows && r < c_end ? __ldcs(C + origin + r * N + c) : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < P; ++u) {
+      const int r = (base + u * THREADS) / BN, c = (base + u * THREADS) % BN;
+      if (c >= cols || r >= rows) continue;
+      const float v = red[(r0 + r) * RS + c];
+      out[origin + r * N + c] = r < c_end ? __fsub_rn(v, cc[u]) : v;
     }
   }
 }
@@ -622,15 +647,16 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, float* __restrict__ out, con
     const int t = threadIdx.x - 64;  // 0..127
     if constexpr (Md::kF16)
       for (int j = t; j < BN; j += 128) col_scale[j] = pow2f(-((n0 + j < N) ? __ldg(w_exp + n0 + j) : 0));
-    if (C && m0 < c_rows && (N & 3) == 0) {
+    if (C && m0 < c_rows) {
       const int rows_per_rank = (BM + splits - 1) / splits;
       const int rank = splits > 1 ? (int)cluster_rank() : 0;
       const int r0 = rank * rows_per_rank, r1 = (r0 + rows_per_rank < BM) ? r0 + rows_per_rank : BM;
       const int64_t ncols = std::min<int64_t>(BN, N - n0);
-      const int lines = (int)ceil_div(ncols * 4, 128);
+      const int lines = (int)ceil_div(ncols * 4 + ((N & 3) != 0 ? 124 : 0), 128);  // a row may start inside a line
       for (int i = t; i < (r1 - r0) * lines; i += 128) {
         const int64_t m = m0 + r0 + i / lines;
-        if (m < M && m < c_rows) prefetch_l2(C + m * N + n0 + (int64_t)(i % lines) * 32);
+        if (m < M && m < c_rows)
+          prefetch_l2(C + m * N + n0 + std::min<int64_t>((int64_t)(i % lines) * 32, ncols - 1));
       }
     }
     pdl_wait();  // the row exponents of A come from the kernel before this one
@@ -757,15 +783,22 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, float* __restrict__ out, con
     const int rank = splits > 1 ? (int)cluster_rank() : 0;
     const int rows_per_rank = (BM + splits - 1) / splits;
     const int r0 = rank * rows_per_rank, r1 = (r0 + rows_per_rank < BM) ? r0 + rows_per_rank : BM;
+    const bool ragged = (N & 3) != 0;
     switch (splits) {
-      case 1: reduce_store<1, BN>(red, r0, r1, m0, n0, M, N, C, out, c_rows); break;
-      case 2: reduce_store<2, BN>(red, r0, r1, m0, n0, M, N, C, out, c_rows); break;
-      case 3: reduce_store<3, BN>(red, r0, r1, m0, n0, M, N, C, out, c_rows); break;
-      case 4: reduce_store<4, BN>(red, r0, r1, m0, n0, M, N, C, out, c_rows); break;
-      case 5: reduce_store<5, BN>(red, r0, r1, m0, n0, M, N, C, out, c_rows); break;
-      case 6: reduce_store<6, BN>(red, r0, r1, m0, n0, M, N, C, out, c_rows); break;
-      case 7: reduce_store<7, BN>(red, r0, r1, m0, n0, M, N, C, out, c_rows); break;
-      default: reduce_store<8, BN>(red, r0, r1, m0, n0, M, N, C, out, c_rows); break;
+      case 1:
+        if (!ragged) reduce_store<1, BN>(red, false, r0, r1, m0, n0, M, N, C, out, c_rows);
+        break;
+      case 2: reduce_store<2, BN>(red, ragged, r0, r1, m0, n0, M, N, C, out, c_rows); break;
+      case 3: reduce_store<3, BN>(red, ragged, r0, r1, m0, n0, M, N, C, out, c_rows); break;
+      case 4: reduce_store<4, BN>(red, ragged, r0, r1, m0, n0, M, N, C, out, c_rows); break;
+      case 5: reduce_store<5, BN>(red, ragged, r0, r1, m0, n0, M, N, C, out, c_rows); break;
+      case 6: reduce_store<6, BN>(red, ragged, r0, r1, m0, n0, M, N, C, out, c_rows); break;
+      case 7: reduce_store<7, BN>(red, ragged, r0, r1, m0, n0, M, N, C, out, c_rows); break;
+      default: reduce_store<8, BN>(red, ragged, r0, r1, m0, n0, M, N, C, out, c_rows); break;
+    }
+    if (ragged) {
+      if (splits > 1) __syncthreads();  // the sums are staged
+      store_ragged<BN>(red, r0, r1, m0, n0, M, N, C, out, c_rows);
     }
   }
   __syncwarp();
@@ -1720,7 +1753,8 @@ TcShape tc_shape_for(int v, int64_t M, int64_t K, int64_t N, int sms, bool f16) 
   return best;
 }
 
-// The cheapest pair form, if it beats `best` (FP16X3): M and N in tiles of the widths, every one unsplit.  rest_tiles counts 128-row tiles, as the other forms do.
+// The cheapest pair form, if it beats `best` (FP16X3): M and N in tiles of the widths, every one unsplit.
+// rest_tiles counts 128-row tiles, as the other forms do.
 void consider_pairs(TcShape& best, int64_t M, int64_t K, int64_t N, double hbm) {
   for (int w = 0; w < kPairs; ++w) {
     const int64_t cols = ceil_div(N, (int64_t)kPair[w].bn), tiles = ceil_div(M, (int64_t)256) * cols;
