@@ -1560,23 +1560,21 @@ int swap_width_index(int64_t tokens) {
   return kSwapWidths - 1;
 }
 
-// The launch variants: tile width, ring size, CTAs per SM, and the cost constants of the launch model
-// below, in us: a round of co-resident CTAs takes F + b K / s (F: setup, pipeline fill, epilogue and
-// cluster reduction; b: the mainloop per 1000 elements of K on FP16X3; TF32X3 takes two k-blocks where
-// FP16X3 takes one).  Fitted to a sweep of every variant, split, persistent and pair form over the eight
-// Llama and Qwen projections at 61 to 2048 rows on GB300 (64 shapes).  Streaming the weight bounds the few-row
-// shapes whatever the form, so no form counts for less than 6 us + its bytes at HBM's rate, and of forms that
-// would stay below that the one with fewer splits is taken (shape_rank).  The picks are within 0.4% of the
-// best form measured on average, 4% at worst; without the HBM term 0.8% and 8% (128 x 2560 by 19456:
-// clusters of 2 43.1 us, unsplit 40.3), and before the MMA issue was fixed 10% on average.
+// The launch variants: tile width, ring size, CTAs per SM, and constants of the launch model (launch_cost) in us:
+// F per round of co-resident CTAs (setup, pipeline fill, epilogue, cluster sum), b per 1000 elements of K.  FP16X3's
+// were fitted to sweeps of every variant, split, persistent and pair form on GB300 over 270 shapes: the eight Llama
+// and Qwen projections at 24 to 2048 rows, and 150 drawn shapes of 17 to 2048 rows, K 64 to 9728 and N to 32768, many
+// of no round size.  The picks are within 0.2 to 0.4% of the best form measured on average over the projections
+// (4.4% at worst) and within 1.7% over the drawn shapes (23%, at 45 us); constants fitted to the projections alone
+// were 8.8% off there and 78% at worst, with pairs for short K and ragged N.  F32 and b32 are TF32X3's.
 struct Variant {
   int bn, rk, cps;
-  double F, b;
+  double F, b, F32, b32;
 };
 constexpr int kVariants = 6;
-constexpr Variant kVariant[kVariants] = {{256, 192, 1, 8.22, 16.08}, {128, 224, 1, 6.26, 10.58},
-                                         {128, 96, 2, 7.33, 17.81},  {160, 224, 1, 6.78, 11.62},
-                                         {192, 224, 1, 7.28, 12.78}, {224, 224, 1, 7.32, 14.40}};
+constexpr Variant kVariant[kVariants] = {{256, 192, 1, 8.03, 15.01, 8.22, 16.08}, {128, 224, 1, 5.66, 9.76, 6.26, 10.58},
+                                         {128, 96, 2, 0.0, 0.0, 7.33, 17.81},     {160, 224, 1, 5.66, 11.62, 6.78, 11.62},
+                                         {192, 224, 1, 7.10, 11.62, 7.28, 12.78}, {224, 224, 1, 6.21, 15.41, 7.32, 14.40}};
 
 // Co-resident clusters of s CTAs of variant v on the current device; clusters must fit inside
 // one GPC, so this is not simply (SMs x CTAs per SM) / s.  Both encodings use the same shared
@@ -1624,8 +1622,7 @@ int max_active_clusters(int v, int s, int sms) {
 
 // Launch shape: a variant, then either one launch with every tile's K split s ways over a cluster, or
 // (TF32X3) whole waves of unsplit tiles followed by the remaining tiles split (so the last wave is not mostly
-// idle), or one persistent launch, on single SMs or on SM pairs.  At least 256 of K per CTA; ties go to
-// the earlier variant and to fewer splits.
+// idle), or one persistent launch, on single SMs or on SM pairs.  At least 64 of K per CTA (TF32X3: 256).
 struct TcShape {
   int v;
   int64_t full_tiles;  // tiles of the first, unsplit launch (whole waves)
@@ -1640,7 +1637,7 @@ struct TcShape {
 // busiest pair b K plus h (the part of a tile's hand-over and epilogue that its successor does not hide).
 // Fitted with the variants above.  A pair beats two single SMs from about 256 rows on: its tile needs
 // 32 KB a k-block per SM where a 128 x 256 tile needs 48, so the tensor pipe is not kept waiting
-// (256-wide: 13.0 against 16.1 us per 1000 of K).  Times at 1024 rows (with the split of A): 3072 by 16384
+// (256-wide: 11.7 against 15.0 us per 1000 of K).  Times at 1024 rows (with the split of A): 3072 by 16384
 // 229 -> 179 us, 3072 by 3072 48 -> 44 us, 8192 by 3072 122 -> 101 us; at 4096 rows 3072 by 16384
 // 871 -> 682 us, where it runs at the power limit (1.8 PFLOP/s of fp16).
 struct PairWidth {
@@ -1648,11 +1645,11 @@ struct PairWidth {
   double F, h, b;
 };
 constexpr int kPairs = 5;
-constexpr PairWidth kPair[kPairs] = {{256, 5.50, 6.96, 13.00},
-                                     {224, 5.33, 3.16, 12.38},
-                                     {192, 4.70, 1.15, 11.25},
-                                     {160, 4.68, 0.00, 10.28},
-                                     {128, 2.68, 1.87, 7.57}};
+constexpr PairWidth kPair[kPairs] = {{256, 5.73, 6.63, 11.70},
+                                     {224, 4.59, 3.66, 11.34},
+                                     {192, 4.60, 1.15, 11.04},
+                                     {160, 5.66, 0.05, 10.90},
+                                     {128, 3.59, 1.87, 7.49}};
 constexpr int kPairRingKb = 448;  // how the test hooks name the pair variants: two SMs' shared memory
 
 // Co-resident pairs of the pair kernel (clusters of two CTAs, one CTA per SM).
@@ -1694,57 +1691,86 @@ int pairs_of(int w) {
   }
 }
 
-// Cost in us of the single-SM persistent form: F once, then per tile of the busiest CTA its mainloop and a
-// hand-over.  It is left where a 256-row tile would be half empty (up to 128 rows of several waves) and for
-// TF32X3.
+// A product as the launch model sees it.  Where a row of an operand is no whole number of 128-byte lines the copies'
+// 64-byte rows (single SMs) straddle lines and take 1.4 times as long, the pairs' 128-byte rows 1.13 times; output
+// rows of no whole 16-byte units go out by single elements (`per_tile` us for 128 rows and columns); and what a round
+// costs besides K is not all spent when a CTA's K is short (below 250: up to `part` of it less).
+struct Problem {
+  int64_t M, K, N;
+  int sms;
+  bool f16;
+  double k_us(double b, double straddle) const { return b * 1e-3 * (double)K * (K % 64 != 0 ? straddle : 1.0); }
+  double ragged_us(double per_tile, int bn) const { return (N & 3) != 0 ? per_tile * bn / 128.0 : 0.0; }
+  double fixed_us(double F, double part, int s) const {
+    return F * (1.0 - part * std::max(0.0, 1.0 - (double)K / (250.0 * s)));
+  }
+};
+constexpr double kStraddle = 1.37, kStraddlePair = 1.13;  // K % 64 != 0
+constexpr double kRagged = 8.8, kRaggedPair = 2.2;        // N % 4 != 0 (and 1.0 for a cluster)
+constexpr double kShort = 0.45, kShortPair = 0.28;
+constexpr double kRound = 4.0;                            // each further round: its start, the tail of the one before
+// The single-SM persistent form: F once, then per tile of the busiest CTA its mainloop and a hand-over.  It is left
+// where a 256-row tile would be half empty (up to 128 rows of several waves) and for TF32X3.
 constexpr double kPersistentTile = 6.73;
 
-double k_cost(double b, int64_t K, bool f16) { return b * 1e-3 * (double)K * (f16 ? 1.0 : 2.0); }
-
-double launch_cost(int v, int64_t tiles, int64_t K, int s, int sms, bool f16) {
+double launch_cost(const Problem& p, int v, int64_t tiles, int s) {
   if (tiles <= 0) return 0.0;
   // clusters of 3, 5 or 7 CTAs: one fewer fits than the occupancy query says (exactly full grids of them
   // took a second round: 256 x 9728 by 2560, 28 clusters of 5, 62 us against 38 for 24 of 5)
-  int64_t clusters = max_active_clusters(v, s, sms);
+  int64_t clusters = max_active_clusters(v, s, p.sms);
   if (s > 1 && (s & 1) != 0 && clusters > 1) --clusters;
-  return (double)ceil_div(tiles, clusters) * (kVariant[v].F + k_cost(kVariant[v].b, K, f16) / (double)s);
+  const double rounds = (double)ceil_div(tiles, clusters);
+  const Variant& w = kVariant[v];
+  if (!p.f16) return rounds * (w.F32 + 2e-3 * w.b32 * (double)p.K / (double)s);
+  const double rows = (double)std::min<int64_t>(p.M, BM) / BM;
+  return (rounds - 1.0) * kRound +
+         rounds * (p.fixed_us(w.F, kShort, s) + p.k_us(w.b, kStraddle) / (double)s +
+                   p.ragged_us(kRagged * rows / s, w.bn) + (s > 1 && (p.N & 3) != 0 ? 1.0 : 0.0));
 }
 
-// What forms are compared by: the cost, not below what HBM allows, and a little per split.
-double shape_rank(double cost, int splits, double hbm) { return std::max(cost, hbm) + 0.1 * splits; }
-double hbm_us(int64_t M, int64_t K, int64_t N, bool f16) {  // 4 or 8 bytes a weight and an entry of A, C in, Y out
-  return 6.0 + ((double)(N + M) * (double)K * (f16 ? 4.0 : 8.0) + 8.0 * (double)M * (double)N) / 6.7e6;
+// What forms are compared by: the cost, not below what HBM allows (4 or 8 bytes a weight and an entry of A, C in, Y
+// out), a little per split, and on FP16X3 a little for the length of the chains of MMAs: of two forms as fast as each
+// other the one that rounds less (a chain truncates at every step; twice its length, up to 1.45 times the error).
+double shape_rank(const Problem& p, double cost, int splits) {
+  const double bytes = (double)(p.N + p.M) * (double)p.K * (p.f16 ? 4.0 : 8.0) + 8.0 * (double)p.M * (double)p.N;
+  if (!p.f16) return std::max(cost, 6.0 + bytes / 6.7e6) + 0.1 * splits;
+  const double chain = (double)std::min<int64_t>(32 * kChainBlocks, round_up(ceil_div(p.K, splits), 32));
+  return std::max(cost, 5.1 + bytes / 6.7e6) + 0.1 * splits + 0.12 * chain / 256.0;
 }
 
-TcShape tc_shape_for(int v, int64_t M, int64_t K, int64_t N, int sms, bool f16) {
-  const double hbm = hbm_us(M, K, N, f16);
+TcShape tc_shape_for(const Problem& p, int v) {
   // the persistent epilogue stores whole float4s: output rows of whole 16-byte units (a launch whose
   // pointers are not 16-byte aligned runs the same tiles unsplit in tc_gemm_kernel: the same sums)
-  const bool persistent_ok = (N & 3) == 0;
-  const int64_t tiles = ceil_div(M, BM) * ceil_div(N, kVariant[v].bn);
-  const int max_s = (int)std::max<int64_t>(1, std::min<int64_t>(MAX_CLUSTER, K / 256));
+  const bool persistent_ok = (p.N & 3) == 0;
+  const int64_t tiles = ceil_div(p.M, BM) * ceil_div(p.N, kVariant[v].bn);
+  const int max_s = (int)std::max<int64_t>(1, std::min<int64_t>(MAX_CLUSTER, p.K / (p.f16 ? 64 : 256)));
   TcShape best{v, 0, tiles, 1, 1e300};
+  // FP16X3 of two CTAs per SM: never more than 4% faster than the other widths, 1.6% slower on average
+  if (p.f16 && kVariant[v].cps > 1) return best;
+  const int64_t wave = max_active_clusters(v, 1, p.sms);
   for (int s = 1; s <= max_s; ++s) {
-    const double c = shape_rank(launch_cost(v, tiles, K, s, sms, f16), s, hbm);
+    if (p.f16 && s > 1 && (s - 1) * round_up(ceil_div(p.K, s), 32) >= p.K) continue;  // a rank without K
+    const double c = shape_rank(p, launch_cost(p, v, tiles, s), s);
     if (c < best.cost * (1.0 - 1e-9)) best = TcShape{v, 0, tiles, s, c};
   }
-  const int64_t wave = max_active_clusters(v, 1, sms);
   // TF32X3: whole waves of unsplit tiles, cut at whole columns of tiles (M is the fast index), so that every
   // output row of a column is summed the same way wherever it sits in M.  FP16X3 leaves such launches to the
   // pairs: a correction cannot follow two orders at once, so the rounding of a product in two launches does
   // not cancel in the unmask (264 x 3072 by 16384: 81 us but 2.4 times the error, 85 us in one launch).
-  const int64_t m_tiles = ceil_div(M, BM);
+  const int64_t m_tiles = ceil_div(p.M, BM);
   const int64_t full = (tiles / wave) * wave / m_tiles * m_tiles, rest = tiles - full;
-  if (!f16 && full > 0 && rest > 0) {
-    const double cf = launch_cost(v, full, K, 1, sms, f16);
+  if (!p.f16 && full > 0 && rest > 0) {
+    const double cf = launch_cost(p, v, full, 1);
     for (int s = 1; s <= max_s; ++s) {
-      const double c = shape_rank(cf + launch_cost(v, rest, K, s, sms, f16), s, hbm);
+      const double c = shape_rank(p, cf + launch_cost(p, v, rest, s), s);
       if (c < best.cost * (1.0 - 1e-9)) best = TcShape{v, full, rest, s, c};
     }
   }
   if (persistent_ok && kVariant[v].cps == 1 && tiles > wave) {  // more than one wave of unsplit tiles
-    const double c = shape_rank(
-        kVariant[v].F + (double)ceil_div(tiles, wave) * (k_cost(kVariant[v].b, K, f16) + kPersistentTile), 1, hbm);
+    const Variant& w = kVariant[v];
+    const double rounds = (double)ceil_div(tiles, wave);
+    const double c = shape_rank(p, p.f16 ? p.fixed_us(w.F, kShort, 1) + rounds * (p.k_us(w.b, kStraddle) + kPersistentTile)
+                                         : w.F32 + rounds * (2e-3 * w.b32 * (double)p.K + kPersistentTile), 1);
     if (c < best.cost * (1.0 - 1e-9)) {
       best = TcShape{v, 0, tiles, 1, c};
       best.persistent = true;
@@ -1753,18 +1779,16 @@ TcShape tc_shape_for(int v, int64_t M, int64_t K, int64_t N, int sms, bool f16) 
   return best;
 }
 
-// The cheapest pair form, if it beats `best` (FP16X3): M and N in tiles of the widths, every one unsplit.
-// rest_tiles counts 128-row tiles, as the other forms do.
-void consider_pairs(TcShape& best, int64_t M, int64_t K, int64_t N, double hbm) {
-  for (int w = 0; w < kPairs; ++w) {
-    const int64_t cols = ceil_div(N, (int64_t)kPair[w].bn), tiles = ceil_div(M, (int64_t)256) * cols;
-    const double c = shape_rank(
-        kPair[w].F + (double)ceil_div(tiles, (int64_t)pairs_of(w)) * (k_cost(kPair[w].b, K, true) + kPair[w].h), 1, hbm);
-    if (c < best.cost * (1.0 - 1e-9)) {
-      best = TcShape{0, 0, ceil_div(M, BM) * cols, 1, c};
-      best.pair = w;
-    }
-  }
+double pair_cost(const Problem& p, int w) {
+  const int64_t tiles = ceil_div(p.M, (int64_t)256) * ceil_div(p.N, (int64_t)kPair[w].bn);
+  return p.fixed_us(kPair[w].F, kShortPair, 1) + (double)ceil_div(tiles, (int64_t)pairs_of(w)) *
+                          (p.k_us(kPair[w].b, kStraddlePair) + kPair[w].h + p.ragged_us(kRaggedPair, kPair[w].bn));
+}
+// The pair form of width w (FP16X3), every tile unsplit.  rest_tiles counts 128-row tiles, as the other forms do.
+TcShape pair_shape(const Problem& p, int w, double cost) {
+  TcShape t{0, 0, ceil_div(p.M, BM) * ceil_div(p.N, (int64_t)kPair[w].bn), 1, cost};
+  t.pair = w;
+  return t;
 }
 
 // k-blocks of a rank of an s-way split of K.
@@ -1778,31 +1802,36 @@ int rank_blocks_of(int64_t K, int s) {
 // tiles with K split seg_splits ways over a cluster, whose rank-order sum is the same fold; or
 // every tile segmented, on single SMs or on pairs.  The cheapest variant and form.
 TcShape tc_bank_shape(int64_t M, int64_t K, int64_t N, int seg_splits, int sms, bool f16) {
+  const Problem p{M, K, N, sms, f16};
   TcShape best{0, 0, 0, 1, 1e300};
   for (int v = 0; v < kVariants; ++v) {
+    if (f16 && kVariant[v].cps > 1) continue;
     const int64_t tiles = ceil_div(M, BM) * ceil_div(N, kVariant[v].bn);
-    const double c = launch_cost(v, tiles, K, 1, sms, f16);
+    const double c = launch_cost(p, v, tiles, 1);
     if (c < best.cost * (1.0 - 1e-9)) best = TcShape{v, 0, tiles, 1, c};
     if (seg_splits < 2 || seg_splits > MAX_CLUSTER) continue;
     const int64_t wave = max_active_clusters(v, 1, sms);
     const int64_t full = (tiles / wave) * wave, rest = tiles - full;
     if (rest == 0) continue;
-    const double c2 = launch_cost(v, full, K, 1, sms, f16) + launch_cost(v, rest, K, seg_splits, sms, f16);
+    const double c2 = launch_cost(p, v, full, 1) + (f16 && full > 0 ? kRound : 0.0) + launch_cost(p, v, rest, seg_splits);
     if (c2 < best.cost * (1.0 - 1e-9)) best = TcShape{v, full, rest, seg_splits, c2};
   }
   // segments longer than a chain belong to ranks that fold chains of their own: only a split reproduces them
   if (f16 && (seg_splits == 1 || rank_blocks_of<Fp16x3>(K, seg_splits) <= kChainBlocks))
-    consider_pairs(best, M, K, N, 0.0);
+    for (int w = 0; w < kPairs; ++w)
+      if (const double c = pair_cost(p, w); c < best.cost * (1.0 - 1e-9)) best = pair_shape(p, w, c);
   return best;
 }
 
 TcShape tc_shape(int64_t M, int64_t K, int64_t N, int sms, bool f16) {
-  TcShape best = tc_shape_for(0, M, K, N, sms, f16);
+  const Problem p{M, K, N, sms, f16};
+  TcShape best = tc_shape_for(p, 0);
   for (int v = 1; v < kVariants; ++v) {
-    const TcShape t = tc_shape_for(v, M, K, N, sms, f16);
+    const TcShape t = tc_shape_for(p, v);
     if (t.cost < best.cost * (1.0 - 1e-9)) best = t;
   }
-  if (f16) consider_pairs(best, M, K, N, hbm_us(M, K, N, f16));
+  for (int w = 0; f16 && w < kPairs; ++w)
+    if (const double c = shape_rank(p, pair_cost(p, w), 1); c < best.cost * (1.0 - 1e-9)) best = pair_shape(p, w, c);
   return best;
 }
 
