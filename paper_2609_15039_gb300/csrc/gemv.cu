@@ -174,35 +174,57 @@ gemv_kernel(float* __restrict__ out, const float* __restrict__ X, const float* _
   const int ksp = staged_ks(MT, ks);
   const int q_row = ksp >> 2, q_len = klen >> 2;
   float* xsf = reinterpret_cast<float*>(xs);
-  // Fused mask: X~ = fl32(X + eta), eta of element (m, k) being lane k % 4 of Philox block (m K + k) / 4 + offset,
-  // as the mask kernel draws it; the blocks of the first row group also write X~ out.  The rows' columns are dealt
-  // out to all threads as one list, so a thread draws MT ks / 1024 of them one after another; with the rows in turn a
-  // slice of 512 columns kept half of the threads idle.
-  const uint64_t off = MASK == kNoMask ? 0ull : nz.offset + (nz.offset_dev ? *nz.offset_dev : 0ull);
-  const bool write_xt = MASK != kNoMask && blockIdx.x == 0;
-  for (int i = threadIdx.x; i < MT * q_row; i += THREADS) {
-    const int m = i / q_row, q = i - m * q_row;
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (m < M && q < q_len) {
-      const bool own = MASK == kNoMask || m < nz.x_rows;  // a row of X (else noise alone, delta blocks further on)
-      if (own) v = __ldg(reinterpret_cast<const float4*>(X + (int64_t)m * K + k0) + q);
-      if constexpr (MASK != kNoMask) {
-        const int64_t mr = own ? m : m - nz.x_rows;
-        const float4 e = draw_block<MASK>((uint64_t)((mr * K + k0) >> 2) + (uint64_t)q + off + (own ? 0ull : nz.delta),
-                                          nz.key, nz.b);
-        v = own ? add4(v, e) : e;
-        if (write_xt) __stcs(reinterpret_cast<float4*>(nz.xt + (int64_t)m * K + k0) + q, v);
-      }
-    }
+  if constexpr (MASK == kNoMask && MT < 8) {
+    auto x4 = [&](int m, int q) {
+      return m < M && q < q_len ? __ldg(reinterpret_cast<const float4*>(X + (int64_t)m * K + k0) + q)
+                                : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
     if constexpr (MT >= 4) {  // rows 2p, 2p + 1 interleaved
-      float* a = xsf + pair_off(m >> 1, ksp, q, 0) + (m & 1);
-      float* b = xsf + pair_off(m >> 1, ksp, q, 1) + (m & 1);
-      a[0] = v.x;
-      a[2] = v.y;
-      b[0] = v.z;
-      b[2] = v.w;
+#pragma unroll
+      for (int p = 0; p < MT / 2; ++p)
+        for (int q = threadIdx.x; q < q_row; q += THREADS) {
+          const float4 a = x4(2 * p, q), b = x4(2 * p + 1, q);
+          *reinterpret_cast<float4*>(xsf + pair_off(p, ksp, q, 0)) = make_float4(a.x, b.x, a.y, b.y);
+          *reinterpret_cast<float4*>(xsf + pair_off(p, ksp, q, 1)) = make_float4(a.z, b.z, a.w, b.w);
+        }
     } else {
-      xs[i] = v;
+#pragma unroll
+      for (int m = 0; m < MT; ++m)
+        for (int q = threadIdx.x; q < q_row; q += THREADS) xs[m * q_row + q] = x4(m, q);
+    }
+  } else {
+    // Fused mask: X~ = fl32(X + eta), eta of element (m, k) being lane k % 4 of Philox block (m K + k) / 4 + offset,
+    // as the mask kernel draws it; the blocks of the first row group also write X~ out.  The rows' columns are dealt
+    // out to all threads as one list, so a thread draws MT ks / 1024 of them one after another; with the rows in turn
+    // a slice of 512 columns kept half of the threads idle.  Without noise to draw, the loops above are faster below 8
+    // rows (two rows' loads in flight, whole float4s stored: a bank of 8 in launches of 4 rows of Llama Q|K|V 20.6 us,
+    // 21.8 as a list) and the list from 8 rows on (64 rows in launches of 8: 116.5 us, 124.9 with the loops).
+    const uint64_t off = MASK == kNoMask ? 0ull : nz.offset + (nz.offset_dev ? *nz.offset_dev : 0ull);
+    const bool write_xt = MASK != kNoMask && blockIdx.x == 0;
+    for (int i = threadIdx.x; i < MT * q_row; i += THREADS) {
+      const int m = i / q_row, q = i - m * q_row;
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (m < M && q < q_len) {
+        const bool own = MASK == kNoMask || m < nz.x_rows;  // a row of X (else noise alone, delta blocks further on)
+        if (own) v = __ldg(reinterpret_cast<const float4*>(X + (int64_t)m * K + k0) + q);
+        if constexpr (MASK != kNoMask) {
+          const int64_t mr = own ? m : m - nz.x_rows;
+          const float4 e = draw_block<MASK>((uint64_t)((mr * K + k0) >> 2) + (uint64_t)q + off + (own ? 0ull : nz.delta),
+                                            nz.key, nz.b);
+          v = own ? add4(v, e) : e;
+          if (write_xt) __stcs(reinterpret_cast<float4*>(nz.xt + (int64_t)m * K + k0) + q, v);
+        }
+      }
+      if constexpr (MT >= 4) {  // rows 2p, 2p + 1 interleaved
+        float* a = xsf + pair_off(m >> 1, ksp, q, 0) + (m & 1);
+        float* b = xsf + pair_off(m >> 1, ksp, q, 1) + (m & 1);
+        a[0] = v.x;
+        a[2] = v.y;
+        b[0] = v.z;
+        b[2] = v.w;
+      } else {
+        xs[i] = v;
+      }
     }
   }
   if constexpr (MASK != kNoMask) load_first();
