@@ -1566,15 +1566,17 @@ int swap_width_index(int64_t tokens) {
 // and Qwen projections at 24 to 2048 rows, and 150 drawn shapes of 17 to 2048 rows, K 64 to 9728 and N to 32768, many
 // of no round size.  The picks are within 0.2 to 0.4% of the best form measured on average over the projections
 // (4.4% at worst) and within 1.7% over the drawn shapes (23%, at 45 us); constants fitted to the projections alone
-// were 8.8% off there and 78% at worst, with pairs for short K and ragged N.  F32 and b32 are TF32X3's.
+// were 8.8% off there and 78% at worst, with pairs for short K and ragged N.  F32 and b32 are
+// TF32X3's, in elements of K of a 256-wide tile, fitted to the projections at 128 to 4096 rows (with FP16X3's constants
+// 200 by 1708 by 5000 took 45.8 us instead of 41.7).
 struct Variant {
   int bn, rk, cps;
   double F, b, F32, b32;
 };
 constexpr int kVariants = 6;
-constexpr Variant kVariant[kVariants] = {{256, 192, 1, 8.03, 15.01, 8.22, 16.08}, {128, 224, 1, 5.66, 9.76, 6.26, 10.58},
-                                         {128, 96, 2, 0.0, 0.0, 7.33, 17.81},     {160, 224, 1, 5.66, 11.62, 6.78, 11.62},
-                                         {192, 224, 1, 7.10, 11.62, 7.28, 12.78}, {224, 224, 1, 6.21, 15.41, 7.32, 14.40}};
+constexpr Variant kVariant[kVariants] = {{256, 192, 1, 8.03, 15.01, 500.0, 1.00}, {128, 224, 1, 5.66, 9.76, 300.0, 1.05},
+                                         {128, 96, 2, 0.0, 0.0, 250.0, 0.95},     {160, 224, 1, 5.66, 11.62, 250.0, 1.05},
+                                         {192, 224, 1, 7.10, 11.62, 300.0, 1.00}, {224, 224, 1, 6.21, 15.41, 550.0, 0.97}};
 
 // Co-resident clusters of s CTAs of variant v on the current device; clusters must fit inside
 // one GPC, so this is not simply (SMs x CTAs per SM) / s.  Both encodings use the same shared
@@ -1628,7 +1630,7 @@ struct TcShape {
   int64_t full_tiles;  // tiles of the first, unsplit launch (whole waves)
   int64_t rest_tiles;  // tiles of the second launch
   int rest_splits;
-  double cost;              // us (shape_rank)
+  double cost;              // shape_rank (us on FP16X3)
   bool persistent = false;  // one launch of tc_persistent_kernel over every tile (unsplit)
   int pair = -1;            // >= 0: width index of tc_pair_kernel, one launch over every tile (unsplit)
 };
@@ -1711,29 +1713,29 @@ constexpr double kShort = 0.45, kShortPair = 0.28;
 constexpr double kRound = 4.0;                            // each further round: its start, the tail of the one before
 // The single-SM persistent form: F once, then per tile of the busiest CTA its mainloop and a hand-over.  It is left
 // where a 256-row tile would be half empty (up to 128 rows of several waves) and for TF32X3.
-constexpr double kPersistentTile = 6.73;
+constexpr double kPersistentTile = 6.73, kPersistentTile32 = 60.0;
 
 double launch_cost(const Problem& p, int v, int64_t tiles, int s) {
   if (tiles <= 0) return 0.0;
+  int64_t clusters = max_active_clusters(v, s, p.sms);
+  const Variant& w = kVariant[v];
+  if (!p.f16) return (double)ceil_div(tiles, clusters) * (w.F32 + 20.0 * s + w.b32 * (double)p.K / (double)s);
   // clusters of 3, 5 or 7 CTAs: one fewer fits than the occupancy query says (exactly full grids of them
   // took a second round: 256 x 9728 by 2560, 28 clusters of 5, 62 us against 38 for 24 of 5)
-  int64_t clusters = max_active_clusters(v, s, p.sms);
   if (s > 1 && (s & 1) != 0 && clusters > 1) --clusters;
   const double rounds = (double)ceil_div(tiles, clusters);
-  const Variant& w = kVariant[v];
-  if (!p.f16) return rounds * (w.F32 + 2e-3 * w.b32 * (double)p.K / (double)s);
   const double rows = (double)std::min<int64_t>(p.M, BM) / BM;
   return (rounds - 1.0) * kRound +
          rounds * (p.fixed_us(w.F, kShort, s) + p.k_us(w.b, kStraddle) / (double)s +
                    p.ragged_us(kRagged * rows / s, w.bn) + (s > 1 && (p.N & 3) != 0 ? 1.0 : 0.0));
 }
 
-// What forms are compared by: the cost, not below what HBM allows (4 or 8 bytes a weight and an entry of A, C in, Y
-// out), a little per split, and on FP16X3 a little for the length of the chains of MMAs: of two forms as fast as each
-// other the one that rounds less (a chain truncates at every step; twice its length, up to 1.45 times the error).
+// What forms are compared by: the cost; on FP16X3 not below what HBM allows (4 bytes a weight and an entry of A, C in,
+// Y out), with a little per split and for the length of the chains of MMAs: of two forms as fast as each other the
+// one that rounds less (a chain truncates at every step; twice its length, up to 1.45 times the error).
 double shape_rank(const Problem& p, double cost, int splits) {
-  const double bytes = (double)(p.N + p.M) * (double)p.K * (p.f16 ? 4.0 : 8.0) + 8.0 * (double)p.M * (double)p.N;
-  if (!p.f16) return std::max(cost, 6.0 + bytes / 6.7e6) + 0.1 * splits;
+  if (!p.f16) return cost;
+  const double bytes = 4.0 * (double)(p.N + p.M) * (double)p.K + 8.0 * (double)p.M * (double)p.N;
   const double chain = (double)std::min<int64_t>(32 * kChainBlocks, round_up(ceil_div(p.K, splits), 32));
   return std::max(cost, 5.1 + bytes / 6.7e6) + 0.1 * splits + 0.12 * chain / 256.0;
 }
@@ -1770,7 +1772,7 @@ TcShape tc_shape_for(const Problem& p, int v) {
     const Variant& w = kVariant[v];
     const double rounds = (double)ceil_div(tiles, wave);
     const double c = shape_rank(p, p.f16 ? p.fixed_us(w.F, kShort, 1) + rounds * (p.k_us(w.b, kStraddle) + kPersistentTile)
-                                         : w.F32 + rounds * (2e-3 * w.b32 * (double)p.K + kPersistentTile), 1);
+                                         : w.F32 + rounds * (w.b32 * (double)p.K + kPersistentTile32), 1);
     if (c < best.cost * (1.0 - 1e-9)) {
       best = TcShape{v, 0, tiles, 1, c};
       best.persistent = true;
