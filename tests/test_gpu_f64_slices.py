@@ -133,3 +133,16 @@ def test_slices_are_closer_than_a_binary64_sum(spl, seed):
         exact = sum(Fraction(a) * Fraction(b) for a, b in zip(X[m].tolist(), W[n].tolist()))
         err.append(float(Fraction(float(got[m, n])) - exact))
     assert math.sqrt(np.mean(np.square(err))) <= U64 * 2.6e8 * 0.02 * math.sqrt(K)
+
+
+def test_smaller_workspace_runs_on_the_fp64_pipe(spl):
+    """A workspace below what the slices take, or none, is not refused where the FP64 pipe's kernel needs less."""
+    M, K, N = 128, 512, 3072
+    g = torch.Generator(device="cuda").manual_seed(9)
+    X = torch.randn((M, K), generator=g, device="cuda")
+    W = torch.randn((N, K), generator=g, device="cuda") * 0.02
+    full = _product(spl, X, W)
+    out = torch.full((M, N), float("nan"), device="cuda", dtype=torch.float64)
+    spl.spl_precompute_noise_product_f64(out, X, W, workspace=None)
+    S = X.double().abs() @ W.double().abs().T
+    assert bool(((out - full).abs() <= 2 * K * U64 / (1 - K * U64) * S).all())
