@@ -23,10 +23,9 @@
 // split keeps fp32's exponent range) or FP32.  W is split once, offline; A is split by a pass before the product
 // into the workspace, so TMA lands every operand tile directly.
 //
-// Products from about 256 rows on run FP16X3 on SM pairs (gemm_pair.cuh).  The others:
-// Kernel shape (one CTA per 128 x BN output tile, 6 warps; BN = 256 with a 192 KB ring and
-// one CTA per SM, or BN = 128 with a 96 KB ring and two CTAs per SM, so that one CTA's
-// epilogue overlaps the other's mainloop):
+// FP16X3 products from about 256 rows on run on SM pairs (gemm_pair.cuh), those of 9 to 16 rows on the swapped
+// kernel (below).  The others: one CTA per 128 x BN output tile, 6 warps; BN = 128 to 256 with a ring of 192 or
+// 224 KB and one CTA per SM, or (TF32X3) BN = 128 with 96 KB and two, one's epilogue beside the other's mainloop:
 //   warp 0      TMA producer: per stage A_hi, A_lo, W_hi, W_lo.
 //   warp 1      TMEM allocator and MMA issuer: per stage 3 products per k-step into one
 //               fp32 accumulator of BN TMEM columns; tcgen05.commit frees the stage.
@@ -36,7 +35,7 @@
 //               subtract C (the fused unmask of Eq. add-and-then-subtract) and store.
 // Every mbarrier wait is bounded (about 1 s of globaltimer); on expiry the kernel raises
 // the device status word, lets issued copies land (again bounded), frees its TMEM and
-// returns.  Role loops run warp-wide (lane 0 issues), so no warp is diverged at a barrier.
+// returns.  Role loops run warp-wide (one elected lane issues), so no warp is diverged at a barrier.
 
 #include <algorithm>
 #include <cmath>
