@@ -302,7 +302,8 @@ tc_f64_kernel(long long* __restrict__ hi, uint32_t* __restrict__ lo, const F64Ro
       mma_commit(drain_bar);  // issued MMAs finish before TMEM is released
     }
     __syncwarp();
-    if (!ok) mbar_wait(drain_bar, 0u, kDrainNs, nullptr);
+    // on the normal path too: the arrival must not land in the shared memory of a CTA that follows this one
+    mbar_wait(drain_bar, 0u, kDrainNs, nullptr);
   } else {
     // ---------------- workers: digits of the tiles into the ring, accumulators into 96-bit sums ----------
     const int tid = (int)threadIdx.x - 32;  // 0 .. F64_WT - 1

@@ -1308,7 +1308,8 @@ tc_swap_kernel(const __grid_constant__ TcMaps maps, float* __restrict__ out, con
       mma_commit(drain_bar);  // issued MMAs finish before TMEM is released
     }
     __syncwarp();
-    if (!ok) mbar_wait(drain_bar, 0u, kDrainNs, nullptr);
+    // on the normal path too: the arrival must not land in the shared memory of a CTA that follows this one
+    mbar_wait(drain_bar, 0u, kDrainNs, nullptr);
   } else {
     // ---------------- warps 2..5: chains summed per piece; pieces out or through the workspace -------
     const int q = warp & 3;  // TMEM lane quarter this warp may access
