@@ -76,7 +76,11 @@ typedef enum spl_path {
 
 /* A weight W[N, K] (fp32, K contiguous) and the splits the tensor-core paths
  * read.  Device pointers owned by the caller; any split may be NULL (the
- * paths that need it then report SPL_EUNSUPPORTED and AUTO skips them). */
+ * paths that need it then report SPL_EUNSUPPORTED and AUTO skips them).
+ * A product starts to read its weight while the calls just before it on the
+ * stream may still run: the splits come from spl_split_tf32 / spl_split_fp16,
+ * which are ordered before it, and w from the caller's own copies or kernels,
+ * not from an output of the preceding call of this library. */
 typedef struct spl_weight {
   const float* w;          /* [N, K] fp32, required */
   const float* tf32_hi;    /* [N, K] from spl_split_tf32 */
@@ -187,7 +191,8 @@ spl_status spl_split_tf32(float* hi, float* lo, const float* src, int64_t count,
  * two e_r (row_exp[r]) that brings the row's largest |entry| into [2^14, 2^15)
  * (0 for an all-zero row); hi + lo = src 2^e_r to about 2^-22 relative.  Done
  * once per weight; hi and lo are [rows, cols] binary16 bit patterns.
- * cols % 8 == 0 (EALIGN otherwise). */
+ * cols % 8 == 0 (EALIGN otherwise).  Complete, in stream order, before any
+ * later call reads the split (a second, empty launch sees to it). */
 spl_status spl_split_fp16(uint16_t* hi, uint16_t* lo, int32_t* row_exp, const float* src, int64_t rows,
                           int64_t cols, cudaStream_t stream);
 

@@ -38,7 +38,8 @@ inline spl_status launch_status() {
 // kernel holds SM resources while waiting on one that is not yet resident, and every tensor-core
 // kernel has its tensor memory before it triggers.  The fp16 split kernels therefore trigger before
 // they wait: the product after a split (at most two kernels ahead) may start loading its weight
-// while the kernel before the split finishes.
+// while the kernel before the split finishes.  The weight itself must be complete by then, so the
+// weight's split (spl_split_fp16) is followed by an empty kernel launched in plain stream order.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -378,6 +378,10 @@ __global__ void __launch_bounds__(kThreads) split_fp16_regs_kernel(uint16_t* __r
   }
 }
 
+// Launched without the dependent-launch attribute it starts when the kernel before it is complete and its writes
+// are visible, so whatever the next kernel reads before its own wait is there.
+__global__ void stream_order_kernel() {}
+
 int grid_for(int64_t work_items, int blocks_per_sm) {
   const int64_t want = ceil_div(work_items, kThreads);
   const int64_t cap = (int64_t)device_sm_count() * blocks_per_sm;
@@ -622,7 +626,14 @@ extern "C" spl_status spl_split_fp16(uint16_t* hi, uint16_t* lo, int32_t* row_ex
   if ((hi && !aligned16(hi)) || (lo && !aligned16(lo)) || (src && !aligned16(src))) return SPL_EALIGN;
   if (cols == 0) return cudaMemsetAsync(row_exp, 0, (size_t)rows * sizeof(int32_t), stream) == cudaSuccess
                             ? SPL_OK : SPL_ECUDA;
-  return run_split_fp16(hi, lo, row_exp, src, rows, cols, stream);
+  const spl_status st = run_split_fp16(hi, lo, row_exp, src, rows, cols, stream);
+  if (st != SPL_OK) return st;
+  // The split may be a weight's, and a product reads its weight before it waits (the product after this call, or the
+  // one after the split of its left operand, both scheduled before this split waits): the split ends here, at the
+  // cost of one empty launch per weight.  (The TF32X3 product's left operand is split by a kernel that waits before
+  // it triggers, so spl_split_tf32 needs none.)
+  stream_order_kernel<<<1, 1, 0, stream>>>();
+  return launch_status();
 }
 
 extern "C" spl_status spl_split_tf32(float* hi, float* lo, const float* src, int64_t count, cudaStream_t stream) {
