@@ -133,6 +133,7 @@ struct Plan {
   int splits;            // K-splits (1 = none)
   int64_t k_per_split;   // multiple of the kernel's K granule
   size_t ws_partials;    // bytes of split partials (at offset kCounterBytes)
+  int swap_ctas;         // CTAs per token tile of the swapped kernel (9-16 rows on FP16X3), else 0
   size_t ws_asplit;      // bytes of the FP16X3 split of A: row exponents, hi, lo (at offset kCounterBytes)
   size_t total() const { return (ws_partials + ws_asplit) ? kCounterBytes + ws_partials + ws_asplit : 0; }
 };

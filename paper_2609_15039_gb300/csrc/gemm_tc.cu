@@ -2025,20 +2025,27 @@ int swap_ctas(int64_t K, int64_t N, int sms) {
   const int64_t even = w_tiles > sms ? sms : std::max<int64_t>(1, std::min<int64_t>(3 * (int64_t)sms / 4, total));
   constexpr int64_t chain = 1024 / SwapCfg<16>::BK;
   const int64_t longest = std::min(chain, 4 * w_tiles >= 3 * (int64_t)sms ? nkb : ceil_div(total, even));
-  const double hbm = (double)total * 32768.0 / 6.7e6;
+  // the two times joined by their 4-norm; every call of 9 to 16 rows runs this, so in products and roots, from the
+  // first k whose chains are short enough on, and only while a larger k can still be better
+  const double hbm = (double)total * 32768.0 / 6.7e6, hbm4 = (hbm * hbm) * (hbm * hbm);
   int64_t best_c = even;
   double best = 1e300;
-  for (int64_t k = 1; k * w_tiles <= sms && k <= nkb; ++k) {
-    const int64_t piece = ceil_div(nkb, k);
-    if (std::min(chain, piece) > longest) continue;
-    const double stream = 0.37 * (double)piece;
-    const double c = std::pow(std::pow(stream, 4.0) + std::pow(hbm, 4.0), 0.25) + (k > 1 ? 2.4 + 0.15 * (double)k : 0.0);
+  for (int64_t k = longest < chain ? ceil_div(nkb, longest) : 1; k * w_tiles <= sms && k <= nkb; ++k) {
+    const double meet = k > 1 ? 2.4 + 0.15 * (double)k : 0.0;
+    if (hbm + meet >= best) break;
+    const double stream = 0.37 * (double)ceil_div(nkb, k), stream2 = stream * stream;
+    const double c = std::sqrt(std::sqrt(stream2 * stream2 + hbm4)) + meet;
     if (c < best * (1.0 - 1e-9)) {
       best = c;
       best_c = k * w_tiles;
     }
   }
   return (int)best_c;
+}
+
+// The same, every CTA with at least one unit.
+int swap_run_ctas(int64_t K, int64_t N, int sms) {
+  return (int)std::min<int64_t>(swap_ctas(K, N, sms), ceil_div(N, BM) * ceil_div(K, (int64_t)SwapCfg<16>::BK));
 }
 
 // Workspace of the swapped kernel's partial tiles: two slots per CTA and token tile of width tn.
@@ -2197,7 +2204,8 @@ Plan plan_tc(int64_t M, int64_t K, int64_t N, int sms, spl_path path) {
   p.kernel = kKernelTc;
   if (tc_swapped(M, path)) {
     p.splits = 1;  // runs of k-blocks, partial tiles summed through the workspace
-    p.ws_partials = tc_partial_bytes(M, K, N, M, path);
+    p.swap_ctas = swap_run_ctas(K, N, sms);
+    p.ws_partials = swap_partial_bytes(M, kSwapTn[swap_width_index(M)], p.swap_ctas);
   } else {
     const TcShape t = tc_shape(M, K, N, sms, path == SPL_PATH_FP16X3);
     p.splits = t.rest_splits;  // partials are reduced through distributed shared memory
@@ -2209,14 +2217,11 @@ Plan plan_tc(int64_t M, int64_t K, int64_t N, int sms, spl_path path) {
 
 size_t tc_partial_bytes(int64_t M, int64_t K, int64_t N, int64_t order_rows, spl_path path) {
   if (!tc_swapped(order_rows, path) || M <= 0 || K <= 0 || N <= 0) return 0;
-  const int64_t total = ceil_div(N, BM) * ceil_div(K, (int64_t)SwapCfg<16>::BK);
-  const int ctas = (int)std::min<int64_t>(swap_ctas(K, N, device_sm_count()), total);
-  return swap_partial_bytes(M, kSwapTn[swap_width_index(M)], ctas);
+  return swap_partial_bytes(M, kSwapTn[swap_width_index(M)], swap_run_ctas(K, N, device_sm_count()));
 }
 
 spl_status run_tc(const LinearArgs& a, const Plan& p) {
-  (void)p;
-  if (tc_swapped(a.M, a.path)) return run_tc_impl(a, -1, -1, 0, 0, 0, false, swap_width_index(a.M));
+  if (tc_swapped(a.M, a.path)) return run_tc_impl(a, -1, -1, 0, 0, 0, false, swap_width_index(a.M), p.swap_ctas);
   return run_tc_impl(a, -1, -1, 0);
 }
 
