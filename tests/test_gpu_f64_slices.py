@@ -20,8 +20,8 @@ def spl():
     return s
 
 
-def _product(spl, X, W):
-    """X W^T through the correction (fp32 X) or through the unmask with C = 0, whose result is rounded to fp32."""
+def _product(spl, X, W, C=None):
+    """X W^T through the correction (fp32 X), or fl32(X W^T - C) through the unmask (binary64 X; C = 0 if not given)."""
     M, K = X.shape
     N = W.shape[0]
     ws = spl.workspace(spl.spl_f64_workspace_bytes(M, K, N))
@@ -32,24 +32,39 @@ def _product(spl, X, W):
         spl.spl_precompute_noise_product_f64(out, X, W, workspace=ws)
     else:
         out = torch.full((M, N), float("nan"), device="cuda")
-        spl.spl_masked_linear_unmask_f64(out, X, W, torch.zeros((M, N), device="cuda", dtype=torch.float64),
-                                         workspace=ws)
+        if C is None:
+            C = torch.zeros((M, N), device="cuda", dtype=torch.float64)
+        spl.spl_masked_linear_unmask_f64(out, X, W, C, workspace=ws)
     assert spl.spl_get_device_status() == 0
     return out
 
 
+def _sums(spl, X, W, exact):
+    """The product's binary64 sums at the outputs of `exact` {(m, n): Fraction}.  Of a binary64 X the entry point
+    returns fl32(sum - C): with C 1024 last places below the exact sum, sum - C is about 1024 of them and every bit
+    of the sum is in the result."""
+    if X.dtype == torch.float32:
+        got = _product(spl, X, W).cpu()
+        assert bool(torch.isfinite(got).all())
+        return {o: Fraction(float(got[o])) for o in exact}
+    C = torch.zeros((X.shape[0], W.shape[0]), dtype=torch.float64)
+    for o, e in exact.items():
+        C[o] = float(e) - 1024 * float(np.spacing(abs(float(e)))) if e else 0.0
+    got = _product(spl, X, W, C.cuda()).cpu()
+    assert bool(torch.isfinite(got).all())
+    return {o: Fraction(float(got[o])) + Fraction(float(C[o])) for o in exact}
+
+
 def _check(spl, X, W, samples):
     X, W = X.cuda(), W.cuda()
-    got = _product(spl, X, W).double().cpu().numpy()
-    assert np.isfinite(got).all()
     K = X.shape[1]
+    exact, S = {}, {}
     for m, n in samples:
         terms = [Fraction(a) * Fraction(b) for a, b in zip(X[m].tolist(), W[n].tolist())]
-        exact, S = sum(terms), float(sum(abs(t) for t in terms))
-        tol = K * U64 / (1 - K * U64) * S + 4 * U64 * abs(float(exact))
-        if X.dtype == torch.float64:
-            tol += 2.0 ** -24 * abs(float(exact)) + 2.0 ** -150  # the result is fp32
-        assert abs(float(Fraction(float(got[m, n])) - exact)) <= tol, (m, n, got[m, n], float(exact), tol)
+        exact[m, n], S[m, n] = sum(terms), float(sum(abs(t) for t in terms))
+    for o, got in _sums(spl, X, W, exact).items():
+        tol = K * U64 / (1 - K * U64) * S[o] + 4 * U64 * abs(float(exact[o])) + 2.0 ** -149  # the least fp32
+        assert abs(float(got - exact[o])) <= tol, (o, float(got), float(exact[o]), tol)
 
 
 def _sample(M, N, count=24):
@@ -69,16 +84,40 @@ def test_slices_match_exact_sums(spl, dtype, M, K, N):
     _check(spl, X.to(dtype), W, _sample(M, N))
 
 
-def test_slices_hold_the_largest_digit_sums(spl):
-    """Every digit at its largest magnitude and of one sign: the accumulators reach their bound, and the sums
-    are exact (53 bits hold them)."""
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+def test_slices_hold_the_largest_digit_sums(spl, dtype):
+    """Digits of the largest magnitude and of one sign all along K, at every place of the weight: binary64 rows whose
+    digits are 64 and six of -128, against fp32 rows whose entries are three digits of -127, placed by the row's one
+    large entry (fp32 X: the same).  Three such pairs meet in an accumulator, as many as 24 bits of weight allow: 3 x
+    128 x 127 x 128 of its 2^24.  All entries are whole in fixed point, so the error is the dropped products (below
+    2^-57.6 of 2^(E_x + E_w) a term) and the result's rounding."""
     M, K, N = 40, 4096, 256
-    x = -float(0x40808080808080) * 2.0 ** -30
-    w = -float(0x408080) * 2.0 ** -40
-    got = _product(spl, torch.full((M, K), x, dtype=torch.float64, device="cuda"),
-                   torch.full((N, K), w, device="cuda"))
-    exact = float(Fraction(x) * Fraction(w) * K)
-    assert torch.equal(got, torch.full_like(got, exact))
+    low = [-float(0x7F7F7F) * 2.0 ** (8 * p - 53) for p in range(4)]  # beside an entry of 1: digits p, p + 1, p + 2
+    W = torch.tensor(low, dtype=torch.float32).repeat(N // 4)[:, None].repeat(1, K)
+    W[:, 0] = 1.0
+    if dtype == torch.float64:
+        X = torch.full((M, K), float(0x3F7F7F7F7F7F80) * 2.0 ** -53, dtype=dtype)  # E = 0
+        X[1::2] *= -2.0 ** 40
+    else:
+        X = torch.tensor(low, dtype=dtype).repeat(M // 4)[:, None].repeat(1, K)
+        X[:, 0] = 1.0
+        X[4:8] *= -2.0 ** 40
+    assert X.unique(dim=0).shape[0] <= 8
+    exact = {}
+    for m in range(8):
+        for n in range(4):
+            exact[m, n] = sum(Fraction(a) * Fraction(b) for a, b in zip(X[m].tolist(), W[n].tolist()))
+    got = _sums(spl, X.cuda(), W.cuda(), exact)
+    for (m, n), g in got.items():
+        scale = 2.0 ** 40 if (m % 2 == 1 if dtype == torch.float64 else m >= 4) else 1.0
+        tol = K * 2.0 ** -57.6 * scale + 2 * U64 * abs(float(exact[m, n]))
+        assert abs(float(g - exact[m, n])) <= tol, (m, n, float(g), float(exact[m, n]))
+    full = _product(spl, X.cuda(), W.cuda())  # every other row and column repeats these, bit for bit
+    period = 2 if dtype == torch.float64 else 8
+    for m in range(M):
+        same = m % period if dtype == torch.float64 else (m if m < 8 else m % 4)
+        assert torch.equal(full[m], full[same])
+    assert torch.equal(full[:, 4:], full[:, :-4])
 
 
 def test_slices_of_rows_that_fixed_point_loses(spl):
