@@ -514,6 +514,12 @@ spl_status spl_test_tc_wait_timeout(float* out, const float* A, const spl_weight
  * occupancy queries. */
 spl_status spl_test_tc_shape(int64_t M, int64_t K, int64_t N, int64_t seg_splits, int64_t* out);
 
+/* Test hook (no counterpart in the paper): *out (host) = the blocks per SM of the
+ * decode kernel's instance for M rows (1..16), a K-slice of ks columns (64..1536)
+ * and mask -1 (none), 0 (Laplace), 1 (Gaussian) or 2 (eps = inf; masked: up to 4
+ * rows).  EINVAL for other arguments or a NULL out. */
+spl_status spl_test_gemv_blocks(int64_t M, int64_t ks, int mask, int64_t* out);
+
 /* Test hook (no counterpart in the paper): *out (host) = the number of clusters
  * of `cluster` CTAs (1..8) of the launch variant (tile_n, ring_kb) -- (256, 192),
  * (128, 224), (128, 96), (160, 224), (192, 224) or (224, 224), or the pair

@@ -123,8 +123,27 @@ struct KernelNoise {
   uint64_t delta;
 };
 
+// The masked instances of a row count keep as many blocks an SM as the unmasked one, for which the plan sizes the
+// grid (3, 2 and 3 at 1, 2 and 4 rows), and the registers that the two buffers of W need.  Left alone, the compiler
+// took 64 to 94 registers for them: instances of 64 held fewer loads in flight, and one row at eps = inf got 2
+// blocks of the 3, a second wave.  us a step of two Llama layers without Down, before and now:
+//   rows                  1     2     4     1 + 1   2 + 2 (a step's rows and the next cycle's)
+//   Laplace   before  115.6 114.2 123.4   113.3   122.8
+//             now     110.9 112.9 122.5   111.5   122.2
+//   Gaussian  before  107.1 132.1 133.3   131.5   132.5
+//             now     107.0 112.3 121.6   111.8   121.0
+//   eps = inf before  133.0 113.2 118.9   111.5   116.7
+//             now     106.6 109.4 118.6   108.4   116.8
+constexpr int masked_blocks(int mt) { return mt == 2 ? 2 : mt == 4 ? 3 : 0; }  // 0: the compiler's choice already
+// One pointer to the lane's rows and their distance instead of a pointer a row: 8 registers.  (One row with Gaussian
+// noise is 109.1 us so, 107.0 with the pointers.)
+constexpr bool one_pointer(int mt, int mask) { return mask != kNoMask && !(mt == 1 && mask == kGaussian); }
+// W's first steps are fetched before the wait: where no noise is drawn meanwhile, which needs the registers (eps = inf
+// 109 -> 106 us at one row and 112 -> 109 at two, but 118 -> 122 at four).
+constexpr bool early_weights(int mt, int mask) { return mask == kNoMask || (mask == kZero && mt <= 2); }
+
 template <int MT, int MASK>
-__global__ void __launch_bounds__(THREADS)
+__global__ void __launch_bounds__(THREADS, MASK == kNoMask ? 0 : masked_blocks(MT))
 gemv_kernel(float* __restrict__ out, const float* __restrict__ X, const float* __restrict__ W,
             const float* __restrict__ C, float* __restrict__ part, unsigned int* __restrict__ counters, int M,
             int64_t K, int64_t N, int ks, int splits, int prefetch_lines, const __grid_constant__ KernelNoise nz,
@@ -147,6 +166,11 @@ gemv_kernel(float* __restrict__ out, const float* __restrict__ X, const float* _
     valid[r] = row0 + 4 * r < N;
     wp[r] = W + (valid[r] ? row0 + 4 * r : 0) * K + k0 + kl;
   }
+  const float* const w0 = W + row0 * K + k0 + kl;
+  const int n_left = (int)std::max<int64_t>(0, std::min<int64_t>(N - row0, 4 * RQ));
+  constexpr bool kOne = one_pointer(MT, MASK), kEarly = early_weights(MT, MASK);
+  auto row_in = [&](int r) { return kOne ? 4 * r < n_left : valid[r]; };
+  auto row_at = [&](int r) { return kOne ? w0 + (int64_t)(4 * r) * K : wp[r]; };
 
   // W never changes, so its first lines are fetched before waiting on the kernel that writes X~
   // and C: the first U steps into registers (after the staging when it draws noise, which needs
@@ -157,14 +181,14 @@ gemv_kernel(float* __restrict__ out, const float* __restrict__ X, const float* _
     for (int u = 0; u < U; ++u)
 #pragma unroll
       for (int r = 0; r < RQ; ++r)
-        w[u][r] = (valid[r] && u * kStep + kl < klen) ? __ldcs(reinterpret_cast<const float4*>(wp[r] + u * kStep))
+        w[u][r] = (row_in(r) && u * kStep + kl < klen) ? __ldcs(reinterpret_cast<const float4*>(row_at(r) + u * kStep))
                                                        : make_float4(0.f, 0.f, 0.f, 0.f);
   };
-  if constexpr (MASK == kNoMask) load_first();
-  for (int l = (MASK == kNoMask ? U : 0) + (lane & 7); l < prefetch_lines && l * kStep < klen; l += 8)
+  if constexpr (kEarly) load_first();
+  for (int l = (kEarly ? U : 0) + (lane & 7); l < prefetch_lines && l * kStep < klen; l += 8)
 #pragma unroll
     for (int r = 0; r < RQ; ++r)
-      if (valid[r]) asm volatile("prefetch.global.L2 [%0];" ::"l"(wp[r] - kl + l * kStep));
+      if (row_in(r)) asm volatile("prefetch.global.L2 [%0];" ::"l"(row_at(r) - kl + l * kStep));
   pdl_wait();
   // the next kernel may be scheduled now: its blocks take the slots this grid leaves free and
   // fetch their first weight lines while this one streams (decode 2.28 -> 2.24 ms per token)
@@ -227,7 +251,7 @@ gemv_kernel(float* __restrict__ out, const float* __restrict__ X, const float* _
       }
     }
   }
-  if constexpr (MASK != kNoMask) load_first();
+  if constexpr (!kEarly) load_first();
   __syncthreads();
 
   float acc[V];
@@ -249,8 +273,8 @@ gemv_kernel(float* __restrict__ out, const float* __restrict__ X, const float* _
       for (int u = 0; u < U; ++u)
 #pragma unroll
         for (int r = 0; r < RQ; ++r)
-          wn[u][r] = (valid[r] && kn + u * kStep + kl < klen)
-                         ? __ldcs(reinterpret_cast<const float4*>(wp[r] + kn + u * kStep))
+          wn[u][r] = (row_in(r) && kn + u * kStep + kl < klen)
+                         ? __ldcs(reinterpret_cast<const float4*>(row_at(r) + kn + u * kStep))
                          : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int u = 0; u < U; ++u) {
@@ -299,8 +323,8 @@ gemv_kernel(float* __restrict__ out, const float* __restrict__ X, const float* _
     for (int u = 0; u < U; ++u)
 #pragma unroll
       for (int r = 0; r < RQ; ++r)
-        wn[u][r] = (valid[r] && kn + u * kStep + kl < klen)
-                       ? __ldcs(reinterpret_cast<const float4*>(wp[r] + kn + u * kStep))
+        wn[u][r] = (row_in(r) && kn + u * kStep + kl < klen)
+                       ? __ldcs(reinterpret_cast<const float4*>(row_at(r) + kn + u * kStep))
                        : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int u = 0; u < U; ++u)
@@ -466,6 +490,16 @@ int blocks_per_sm(int mt, int64_t ks) {
   return v;
 }
 
+// The instance for `mask` (kNoMask, or a mechanism) at a padded row count, null where there is none.
+void* instance_for(int mt, int mask) {
+  if (mask == kNoMask) return kernel_for(mt);
+  if (mt > kGemvMaskMaxM || mask < kLaplace || mask > kZero) return nullptr;
+  void* const masked[3][3] = {{kernel_ptr<1, kLaplace>(), kernel_ptr<1, kGaussian>(), kernel_ptr<1, kZero>()},
+                              {kernel_ptr<2, kLaplace>(), kernel_ptr<2, kGaussian>(), kernel_ptr<2, kZero>()},
+                              {kernel_ptr<4, kLaplace>(), kernel_ptr<4, kGaussian>(), kernel_ptr<4, kZero>()}};
+  return masked[mt == 1 ? 0 : mt == 2 ? 1 : 2][mask];
+}
+
 }  // namespace
 
 int64_t gemv_max_ks(int64_t M) {
@@ -628,4 +662,20 @@ extern "C" spl_status spl_masked_linear_unmask_noalloc(float* Y, const float* Xt
   args.c_rows = M;
   args.path = SPL_PATH_FP32;
   return run_gemv(args, plan);
+}
+
+// Test hook: resident blocks per SM of the decode kernel's instance for M rows, a K-slice of ks columns and `mask` (-1:
+// none; 0 Laplace, 1 Gaussian, 2 eps = inf).  No GPU work; needs a current CUDA device for the occupancy query.
+extern "C" spl_status spl_test_gemv_blocks(int64_t M, int64_t ks, int mask, int64_t* out) {
+  using namespace spl;
+  if (!out || M < 1 || M > kGemvMaxM || ks < kSliceAlign || ks > kMaxKs) return SPL_EINVAL;
+  const int mt = padded_m(M);
+  void* const kernel = instance_for(mt, mask);
+  if (!kernel) return SPL_EINVAL;
+  if (!smem_attr_set()) return SPL_ECUDA;
+  int n = 0;
+  const size_t smem = (size_t)mt * staged_ks(mt, (int)ks) * sizeof(float);
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, THREADS, smem) != cudaSuccess) return SPL_ECUDA;
+  *out = n;
+  return SPL_OK;
 }

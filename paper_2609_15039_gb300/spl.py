@@ -92,6 +92,7 @@ _SIGS = {
     "spl_choose_path": (_I, [ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_double), _P, _P, _PW, _I64,
                              _I64, _I64, _P, _SZ, _P]),
     "spl_test_tc_wait_timeout": (_I, [_P, _P, _PW, _I64, _I64, _I64, _P, _SZ, _P]),
+    "spl_test_gemv_blocks": (_I, [_I64, _I64, _I, ctypes.POINTER(ctypes.c_int64)]),
     "spl_test_tc_capacity": (_I, [_I64, _I64, _I64, ctypes.POINTER(ctypes.c_int64)]),
     "spl_test_tc_shape": (_I, [_I64, _I64, _I64, _I64, ctypes.POINTER(ctypes.c_int64)]),
     "spl_test_tc_product": (_I, [_P, _P, _PW, _P, _I64, _I64, _I64, _I, _I, _I, _I, _I64, _I, _I, _P, _SZ, _P]),
@@ -653,6 +654,13 @@ def spl_test_tc_shape(M, K, N, seg_splits=0):
     out = (ctypes.c_int64 * 6)()
     _check(lib().spl_test_tc_shape(int(M), int(K), int(N), int(seg_splits), out), "spl_test_tc_shape")
     return tuple(int(v) for v in out)
+
+
+def spl_test_gemv_blocks(M, ks, mask=-1):
+    """Resident blocks per SM of the decode kernel's instance (mask: -1 none, 0 Laplace, 1 Gaussian, 2 eps = inf)."""
+    out = ctypes.c_int64(0)
+    _check(lib().spl_test_gemv_blocks(int(M), int(ks), int(mask), ctypes.byref(out)), "spl_test_gemv_blocks")
+    return int(out.value)
 
 
 def spl_test_tc_capacity(tile_n, ring_kb, cluster):
