@@ -127,6 +127,19 @@ __device__ __forceinline__ int fp16_row_exponent(float amax) {
   return s < -126 ? -126 : (s > 126 ? 126 : s);
 }
 
+// Launch shape of a tcgen05 product (gemm_tc.cu): a variant, then either one launch with every tile's K split s ways
+// over a cluster, or (TF32X3) whole waves of unsplit tiles followed by the remaining tiles split (so the last wave is
+// not mostly idle), or one persistent launch, on single SMs or on SM pairs.  At least 64 of K per CTA (TF32X3: 256).
+struct TcShape {
+  int v;
+  int64_t full_tiles;  // tiles of the first, unsplit launch (whole waves)
+  int64_t rest_tiles;  // tiles of the second launch
+  int rest_splits;
+  double cost;              // shape_rank (us on FP16X3)
+  bool persistent = false;  // one launch of tc_persistent_kernel over every tile (unsplit)
+  int pair = -1;            // >= 0: width index of tc_pair_kernel, one launch over every tile (unsplit)
+};
+
 // Split-K plans: how many K-splits each kernel uses and the workspace it needs.
 struct Plan {
   int kernel;            // 0 = GEMV (decode), 1 = FP32 SIMT GEMM, 2 = tcgen05 GEMM (TF32X3 / FP16X3)
@@ -134,6 +147,7 @@ struct Plan {
   int64_t k_per_split;   // multiple of the kernel's K granule
   size_t ws_partials;    // bytes of split partials (at offset kCounterBytes)
   int swap_ctas;         // CTAs per token tile of the swapped kernel (9-16 rows on FP16X3), else 0
+  TcShape tc;            // the other tcgen05 kernels' launch shape
   size_t ws_asplit;      // bytes of the FP16X3 split of A: row exponents, hi, lo (at offset kCounterBytes)
   size_t total() const { return (ws_partials + ws_asplit) ? kCounterBytes + ws_partials + ws_asplit : 0; }
 };
@@ -164,12 +178,12 @@ spl_status run_gemv_masked(const LinearArgs& a, const Plan& p, const MaskNoise& 
 // Argument check shared by the noise entries.
 spl_status validate_noise(int64_t rows, int64_t cols, double sensitivity, double eps, spl_mech mech);
 int64_t gemv_max_ks(int64_t M);                           // largest K-slice the decode kernel stages for M rows
-// Launch variant and K-split of a one-launch tcgen05 call (false if the call makes two launches);
-// variant -1 is the swapped kernel of few rows.
-bool tc_uniform_shape(int64_t M, int64_t K, int64_t N, spl_path path, int* variant, int* splits);
-// A tcgen05 product whose every output is summed in the order the masked product of `order_rows`
-// rows uses (the correction bank): the same K ranges, accumulation chains and cluster order.
-spl_status run_tc_matched(const LinearArgs& a, int64_t order_rows);
+// K-split of a planned tcgen05 call of one launch (1 for the swapped kernel of few rows); 0 if it makes two.
+int tc_uniform_splits(const Plan& p);
+// A tcgen05 product whose every output is summed in the order of the masked product that was planned with
+// tc_uniform_splits `splits` and `swap_ctas` (the correction bank): the same K ranges, accumulation chains and
+// cluster order.
+spl_status run_tc_matched(const LinearArgs& a, int splits, int swap_ctas);
 size_t tc_asplit_bytes(int64_t M, int64_t K, spl_path path);  // FP16X3 split of A in the workspace (0 for TF32X3)
 // Workspace for the partial tiles of a tcgen05 product of M rows summed in the order of `order_rows`
 // (the swapped kernel's runs; 0 for the cluster-reduced kernels), after the split of A.

@@ -77,6 +77,16 @@ constexpr int MAX_CLUSTER = 8;                         // split-K CTAs of one ou
 // the running sum with a round-to-nearest fp32 add (R = fl(R + P)), so the bias of every chain is
 // bounded whatever K is, and the folds' own errors are unbiased.  A fold costs ~0.35 us per CTA.
 constexpr int kChainBlocks = 32;
+// FP16X3 tiles whose K is not split: chains of 512 elements.  The error of a correction then halves (at K = 3072
+// 3.6e-6 -> 1.8e-6 of the result's norm, against 64 bits; a K-split over 3, 4, 5 or 6 CTAs has 3.6, 2.7, 2.2 and
+// 1.8e-6), and on pairs, which fold in registers beside the MMAs, it costs at most 1%: 1024 x 3072 by 16384 175.2 ->
+// 175.7 us, by 5120 67.0 -> 67.8 (chains of 256: 181.3 and 71.9).  Single SMs fold in TMEM while the MMAs wait: 61 x
+// 2560 by 19456, which HBM bounds, 39.5 -> 39.7 us; 128 x 3072 by 5120 unsplit 38.8 -> 40.0.
+constexpr int kUnsplitBlocks = 16;
+template <class Md>
+constexpr int chain_blocks(int splits) {  // longest chain of a CTA whose K is split `splits` ways
+  return Md::kF16 && splits == 1 ? kUnsplitBlocks : kChainBlocks;
+}
 constexpr uint32_t AUX_BYTES = 2048;                   // barriers, TMEM slot, abort flag; column scales at +1024
 
 // ---- instruction descriptors (tcgen05.mma kind::tf32 / kind::f16) ---------------
@@ -1622,19 +1632,6 @@ int max_active_clusters(int v, int s, int sms) {
   return c;
 }
 
-// Launch shape: a variant, then either one launch with every tile's K split s ways over a cluster, or
-// (TF32X3) whole waves of unsplit tiles followed by the remaining tiles split (so the last wave is not mostly
-// idle), or one persistent launch, on single SMs or on SM pairs.  At least 64 of K per CTA (TF32X3: 256).
-struct TcShape {
-  int v;
-  int64_t full_tiles;  // tiles of the first, unsplit launch (whole waves)
-  int64_t rest_tiles;  // tiles of the second launch
-  int rest_splits;
-  double cost;              // shape_rank (us on FP16X3)
-  bool persistent = false;  // one launch of tc_persistent_kernel over every tile (unsplit)
-  int pair = -1;            // >= 0: width index of tc_pair_kernel, one launch over every tile (unsplit)
-};
-
 // Widths of the pair kernel's 256-row tiles (FP16X3) and their cost in us: F once, then per tile of the
 // busiest pair b K plus h (the part of a tile's hand-over and epilogue that its successor does not hide).
 // Fitted with the variants above.  A pair beats two single SMs from about 256 rows on: its tile needs
@@ -1711,6 +1708,13 @@ constexpr double kStraddle = 1.37, kStraddlePair = 1.13;  // K % 64 != 0
 constexpr double kRagged = 8.8, kRaggedPair = 2.2;        // N % 4 != 0 (and 1.0 for a cluster)
 constexpr double kShort = 0.45, kShortPair = 0.28;
 constexpr double kRound = 4.0;                            // each further round: its start, the tail of the one before
+// Folds beyond those of chains of kChainBlocks (with which the constants were fitted), us each and round: in TMEM, in
+// TMEM beside the next tile's MMAs, in registers beside them.
+constexpr double kFold = 0.35, kFoldPersistent = 0.8, kFoldPair = 0.13;
+int more_folds(int64_t K) {
+  const int64_t nkb = ceil_div(K, (int64_t)32);
+  return (int)(ceil_div(nkb, (int64_t)kUnsplitBlocks) - ceil_div(nkb, (int64_t)kChainBlocks));
+}
 // The single-SM persistent form: F once, then per tile of the busiest CTA its mainloop and a hand-over.  It is left
 // where a 256-row tile would be half empty (up to 128 rows of several waves) and for TF32X3.
 constexpr double kPersistentTile = 6.73, kPersistentTile32 = 60.0;
@@ -1726,21 +1730,53 @@ double launch_cost(const Problem& p, int v, int64_t tiles, int s) {
   const double rounds = (double)ceil_div(tiles, clusters);
   const double rows = (double)std::min<int64_t>(p.M, BM) / BM;
   return (rounds - 1.0) * kRound +
-         rounds * (p.fixed_us(w.F, kShort, s) + p.k_us(w.b, kStraddle) / (double)s +
+         rounds * (p.fixed_us(w.F, kShort, s) + p.k_us(w.b, kStraddle) / (double)s + (s == 1 ? kFold * more_folds(p.K) : 0.0) +
                    p.ragged_us(kRagged * rows / s, w.bn) + (s > 1 && (p.N & 3) != 0 ? 1.0 : 0.0));
 }
 
 // What forms are compared by: the cost; on FP16X3 not below what HBM allows (4 bytes a weight and an entry of A, C in,
 // Y out), with a little per split and for the length of the chains of MMAs: of two forms as fast as each other the
-// one that rounds less (a chain truncates at every step; twice its length, up to 1.45 times the error).
+// one that rounds less.
 double shape_rank(const Problem& p, double cost, int splits) {
   if (!p.f16) return cost;
   const double bytes = 4.0 * (double)(p.N + p.M) * (double)p.K + 8.0 * (double)p.M * (double)p.N;
-  const double chain = (double)std::min<int64_t>(32 * kChainBlocks, round_up(ceil_div(p.K, splits), 32));
+  const int64_t longest = 32 * chain_blocks<Fp16x3>(splits);
+  const double chain = (double)std::min<int64_t>(longest, round_up(ceil_div(p.K, splits), 32));
   return std::max(cost, 5.1 + bytes / 6.7e6) + 0.1 * splits + 0.12 * chain / 256.0;
 }
 
-TcShape tc_shape_for(const Problem& p, int v) {
+// Square of an FP16X3 form's rounding error, up to a constant: a chain of length L truncates in proportion to L times
+// its own size (a square root of L), so the chains' L^3 add up.  Measured against 64 bits at K = 2560 to 4096 over
+// splits of 1 to 8 ways and chains of 256 to 1024, the error is 3.6e-9 sqrt(error2) within 2%.
+double error2(int64_t K, int splits, int chain) {
+  const int64_t kps = round_up(ceil_div(K, splits), 32);
+  double sum = 0.0;
+  for (int64_t k0 = 0; k0 < K; k0 += kps) {
+    const int64_t len = std::min(kps, K - k0), rest = len % chain;
+    sum += (double)(len / chain) * chain * chain * chain + (double)rest * rest * rest;
+  }
+  return sum / (double)K;
+}
+// No FP16X3 form may round more than this: the error of the form that the model of single SMs (TF32X3's: as many
+// splits as fill the chip) takes, with chains of kChainBlocks.  It decides where a split of K would be faster with
+// longer chains, which it must not buy: 128 x 3072 by 5120 19.0 us split 4 ways (2.7e-6), 20.2 us 5 ways (2.2e-6); 61 x
+// 4096 by 2560 15.0 us 6 ways (2.4e-6), 15.3 us 8 ways (1.8e-6).
+TcShape tc_shape_for(const Problem& p, int v, double max_error2 = 1e300);
+double error2_limit(const Problem& p) {
+  Problem q = p;
+  q.f16 = false;
+  TcShape t = tc_shape_for(q, 0);
+  for (int v = 1; v < kVariants; ++v) {
+    const TcShape u = tc_shape_for(q, v);
+    if (u.cost < t.cost * (1.0 - 1e-9)) t = u;
+  }
+  const double full = (double)t.full_tiles, rest = (double)t.rest_tiles;
+  return (full * error2(p.K, 1, 32 * kChainBlocks) + rest * error2(p.K, t.rest_splits, 32 * kChainBlocks)) / (full + rest) *
+         (1.0 + 1e-9);
+}
+double unsplit_error2(int64_t K) { return error2(K, 1, 32 * kUnsplitBlocks); }
+
+TcShape tc_shape_for(const Problem& p, int v, double max_error2) {
   // the persistent epilogue stores whole float4s: output rows of whole 16-byte units (a launch whose
   // pointers are not 16-byte aligned runs the same tiles unsplit in tc_gemm_kernel: the same sums)
   const bool persistent_ok = (p.N & 3) == 0;
@@ -1752,6 +1788,7 @@ TcShape tc_shape_for(const Problem& p, int v) {
   const int64_t wave = max_active_clusters(v, 1, p.sms);
   for (int s = 1; s <= max_s; ++s) {
     if (p.f16 && s > 1 && (s - 1) * round_up(ceil_div(p.K, s), 32) >= p.K) continue;  // a rank without K
+    if (p.f16 && (s == 1 ? unsplit_error2(p.K) : error2(p.K, s, 32 * kChainBlocks)) > max_error2) continue;
     const double c = shape_rank(p, launch_cost(p, v, tiles, s), s);
     if (c < best.cost * (1.0 - 1e-9)) best = TcShape{v, 0, tiles, s, c};
   }
@@ -1768,10 +1805,12 @@ TcShape tc_shape_for(const Problem& p, int v) {
       if (c < best.cost * (1.0 - 1e-9)) best = TcShape{v, full, rest, s, c};
     }
   }
-  if (persistent_ok && kVariant[v].cps == 1 && tiles > wave) {  // more than one wave of unsplit tiles
+  if (persistent_ok && kVariant[v].cps == 1 && tiles > wave &&  // more than one wave of unsplit tiles
+      (!p.f16 || unsplit_error2(p.K) <= max_error2)) {
     const Variant& w = kVariant[v];
     const double rounds = (double)ceil_div(tiles, wave);
-    const double c = shape_rank(p, p.f16 ? p.fixed_us(w.F, kShort, 1) + rounds * (p.k_us(w.b, kStraddle) + kPersistentTile)
+    const double c = shape_rank(p, p.f16 ? p.fixed_us(w.F, kShort, 1) + rounds * (p.k_us(w.b, kStraddle) + kPersistentTile +
+                                                                                         kFoldPersistent * more_folds(p.K))
                                          : w.F32 + rounds * (w.b32 * (double)p.K + kPersistentTile32), 1);
     if (c < best.cost * (1.0 - 1e-9)) {
       best = TcShape{v, 0, tiles, 1, c};
@@ -1784,7 +1823,8 @@ TcShape tc_shape_for(const Problem& p, int v) {
 double pair_cost(const Problem& p, int w) {
   const int64_t tiles = ceil_div(p.M, (int64_t)256) * ceil_div(p.N, (int64_t)kPair[w].bn);
   return p.fixed_us(kPair[w].F, kShortPair, 1) + (double)ceil_div(tiles, (int64_t)pairs_of(w)) *
-                          (p.k_us(kPair[w].b, kStraddlePair) + kPair[w].h + p.ragged_us(kRaggedPair, kPair[w].bn));
+                          (p.k_us(kPair[w].b, kStraddlePair) + kPair[w].h + p.ragged_us(kRaggedPair, kPair[w].bn) +
+                           kFoldPair * more_folds(p.K));
 }
 // The pair form of width w (FP16X3), every tile unsplit.  rest_tiles counts 128-row tiles, as the other forms do.
 TcShape pair_shape(const Problem& p, int w, double cost) {
@@ -1827,35 +1867,40 @@ TcShape tc_bank_shape(int64_t M, int64_t K, int64_t N, int seg_splits, int sms, 
 
 TcShape tc_shape(int64_t M, int64_t K, int64_t N, int sms, bool f16) {
   const Problem p{M, K, N, sms, f16};
-  TcShape best = tc_shape_for(p, 0);
-  for (int v = 1; v < kVariants; ++v) {
-    const TcShape t = tc_shape_for(p, v);
-    if (t.cost < best.cost * (1.0 - 1e-9)) best = t;
+  double limit = f16 ? error2_limit(p) : 1e300;
+  for (;;) {
+    TcShape best = tc_shape_for(p, 0, limit);
+    for (int v = 1; v < kVariants; ++v) {
+      const TcShape t = tc_shape_for(p, v, limit);
+      if (t.cost < best.cost * (1.0 - 1e-9)) best = t;
+    }
+    for (int w = 0; f16 && unsplit_error2(K) <= limit && w < kPairs; ++w)
+      if (const double c = shape_rank(p, pair_cost(p, w), 1); c < best.cost * (1.0 - 1e-9)) best = pair_shape(p, w, c);
+    if (best.cost < 1e299) return best;
+    limit = 1e300;  // not met: the limit's own form is among those above or rounds more than the unsplit one
   }
-  for (int w = 0; f16 && w < kPairs; ++w)
-    if (const double c = shape_rank(p, pair_cost(p, w), 1); c < best.cost * (1.0 - 1e-9)) best = pair_shape(p, w, c);
-  return best;
 }
 
-// Segments of a CTA whose K range is k_range elements: kChainBlocks when the range is longer, else 0
+// Segments of a CTA whose K range, one of `splits`, is k_range elements: chain_blocks when it is longer, else 0
 // (one chain).
 template <class Md>
-int chain_segments(int64_t k_range) {
-  return ceil_div(k_range, (int64_t)Md::BK) > kChainBlocks ? kChainBlocks : 0;
+int chain_segments(int64_t k_range, int splits) {
+  const int chain = chain_blocks<Md>(splits);
+  return ceil_div(k_range, (int64_t)Md::BK) > chain ? chain : 0;
 }
 
 template <class Md, int BN, int RK>
 spl_status launch_tc(const LinearArgs& a, const uint16_t* a_hi, const uint16_t* a_lo, const int* a_exp,
                      TcShape shape, int skip_kblock, int seg_splits) {
-  // Every CTA cuts its K range into chains of at most kChainBlocks k-blocks.  A correction in the
+  // Every CTA cuts its K range into chains of at most chain_blocks k-blocks.  A correction in the
   // order of a seg_splits-way split (seg_splits > 0, the bank) reproduces, per tile, what the online
   // product did: an online split of at most kChainBlocks k-blocks per rank is one chain per rank,
   // summed in rank order, which one CTA over all of K reproduces by folding segments cut at the
-  // split's boundaries; an unsplit online product (seg_splits = 1) is folded at kChainBlocks; an
+  // split's boundaries; an unsplit online product (seg_splits = 1) is folded at chain_blocks(1); an
   // online split whose ranks fold chains of their own is reproduced by the same cluster split.
   int seg_blocks = 0;  // segments of the unsplit tiles of a seg_splits launch
   if (seg_splits == 1) {
-    seg_blocks = chain_segments<Md>(a.K);
+    seg_blocks = chain_segments<Md>(a.K, 1);
   } else if (seg_splits > 1) {
     const int rank_blocks = rank_blocks_of<Md>(a.K, seg_splits);
     if (rank_blocks <= kChainBlocks) {
@@ -1904,8 +1949,8 @@ spl_status launch_tc(const LinearArgs& a, const uint16_t* a_hi, const uint16_t* 
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, tc_persistent_kernel<Md, BN, RK>, maps, a.out, a.c, a_exp,
-                                             (const int*)a.w_exp, a.M, a.K, a.N, (int)tiles, m_tiles, kChainBlocks,
-                                             a.c_rows);
+                                             (const int*)a.w_exp, a.M, a.K, a.N, (int)tiles, m_tiles,
+                                             chain_blocks<Md>(1), a.c_rows);
     note_launches(1);
     return e == cudaSuccess ? SPL_OK : SPL_ECUDA;
   }
@@ -1916,7 +1961,7 @@ spl_status launch_tc(const LinearArgs& a, const uint16_t* a_hi, const uint16_t* 
   auto launch = [&](int64_t tiles, int64_t base, int splits, int seg) -> spl_status {
     if (tiles <= 0) return SPL_OK;
     const int64_t kps = round_up(ceil_div(a.K, splits), Md::BK);
-    if (seg == 0) seg = chain_segments<Md>(kps);  // chains of at most kChainBlocks within the CTA's range
+    if (seg == 0) seg = chain_segments<Md>(kps, splits);
     cudaLaunchConfig_t cfg;
     std::memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3((unsigned)tiles, 1, (unsigned)splits);
@@ -2107,9 +2152,10 @@ spl_status launch_swap(const LinearArgs& a, const uint16_t* x_hi, const uint16_t
 // (0: the library's count, which depends on K and N only, so a bank of any width meets the online
 // product's runs).
 // pair_w >= 0: every tile on the pair kernel of that width index (FP16X3).
+// planned: the launch shape, where the caller has it (else it is worked out here).
 spl_status run_tc_impl(const LinearArgs& a, int skip_kblock, int forced_v, int forced_splits, int seg_splits = 0,
                        int64_t forced_full = 0, bool forced_persistent = false, int swap_w = -1, int swap_s = 0,
-                       int pair_w = -1) {
+                       int pair_w = -1, const TcShape* planned = nullptr) {
   const int cc = device_cc();
   if (cc != 100 && cc != 103) return SPL_EUNSUPPORTED;
   const bool f16 = a.path == SPL_PATH_FP16X3;
@@ -2173,14 +2219,14 @@ spl_status run_tc_impl(const LinearArgs& a, int skip_kblock, int forced_v, int f
   } else if (seg_splits > 0) {
     shape = tc_bank_shape(a.M, a.K, a.N, seg_splits, device_sm_count(), f16);
   } else {
-    shape = tc_shape(a.M, a.K, a.N, device_sm_count(), f16);
+    shape = planned ? *planned : tc_shape(a.M, a.K, a.N, device_sm_count(), f16);
   }
   if (pair_w >= 0) shape.pair = pair_w;
   const uint16_t* hi = static_cast<const uint16_t*>(a_hi);
   const uint16_t* lo = static_cast<const uint16_t*>(a_lo);
   if (f16 && shape.pair >= 0 && skip_kblock < 0) {
-    // segments at the online split's K ranges where each is one chain, else chains of kChainBlocks
-    int chain = kChainBlocks;
+    // segments at the online split's K ranges where each is one chain, else the unsplit form's chains
+    int chain = chain_blocks<Fp16x3>(1);
     if (seg_splits > 1) chain = rank_blocks_of<Fp16x3>(a.K, seg_splits);
     if (chain > kChainBlocks) return SPL_EINVAL;
     return launch_pair(a, hi, lo, a_exp, shape.pair, chain);
@@ -2207,8 +2253,8 @@ Plan plan_tc(int64_t M, int64_t K, int64_t N, int sms, spl_path path) {
     p.swap_ctas = swap_run_ctas(K, N, sms);
     p.ws_partials = swap_partial_bytes(M, kSwapTn[swap_width_index(M)], p.swap_ctas);
   } else {
-    const TcShape t = tc_shape(M, K, N, sms, path == SPL_PATH_FP16X3);
-    p.splits = t.rest_splits;  // partials are reduced through distributed shared memory
+    p.tc = tc_shape(M, K, N, sms, path == SPL_PATH_FP16X3);
+    p.splits = p.tc.rest_splits;  // partials are reduced through distributed shared memory
   }
   p.k_per_split = ceil_div(K, p.splits);
   p.ws_asplit = tc_asplit_bytes(M, K, path);
@@ -2222,27 +2268,18 @@ size_t tc_partial_bytes(int64_t M, int64_t K, int64_t N, int64_t order_rows, spl
 
 spl_status run_tc(const LinearArgs& a, const Plan& p) {
   if (tc_swapped(a.M, a.path)) return run_tc_impl(a, -1, -1, 0, 0, 0, false, swap_width_index(a.M), p.swap_ctas);
-  return run_tc_impl(a, -1, -1, 0);
+  return run_tc_impl(a, -1, -1, 0, 0, 0, false, -1, 0, -1, &p.tc);
 }
 
-bool tc_uniform_shape(int64_t M, int64_t K, int64_t N, spl_path path, int* variant, int* splits) {
-  if (tc_swapped(M, path)) {  // one launch of the swapped kernel
-    *variant = -1;
-    *splits = 1;
-    return true;
-  }
-  const TcShape t = tc_shape(M, K, N, device_sm_count(), path == SPL_PATH_FP16X3);
-  if (t.full_tiles > 0 && t.rest_tiles > 0) return false;
-  *variant = t.pair >= 0 ? kVariants + t.pair : t.v;
-  *splits = t.full_tiles > 0 ? 1 : t.rest_splits;
-  return true;
+int tc_uniform_splits(const Plan& p) {
+  if (p.swap_ctas > 0) return 1;  // one launch of the swapped kernel
+  if (p.tc.full_tiles > 0 && p.tc.rest_tiles > 0) return 0;
+  return p.tc.full_tiles > 0 ? 1 : p.tc.rest_splits;
 }
 
-spl_status run_tc_matched(const LinearArgs& a, int64_t order_rows) {
-  if (tc_swapped(order_rows, a.path))  // the swapped kernel with the online runs; a width for all of M
-    return run_tc_impl(a, -1, -1, 0, 0, 0, false, swap_width_index(a.M), 0);
-  int variant = 0, splits = 1;
-  if (!tc_uniform_shape(order_rows, a.K, a.N, a.path, &variant, &splits)) return SPL_EINVAL;
+spl_status run_tc_matched(const LinearArgs& a, int splits, int swap_ctas) {
+  if (swap_ctas > 0)  // the swapped kernel with the online runs; a width for all of M
+    return run_tc_impl(a, -1, -1, 0, 0, 0, false, swap_width_index(a.M), swap_ctas);
   if (splits < 1 || splits > MAX_CLUSTER) return SPL_ESHAPE;
   return run_tc_impl(a, -1, -1, 0, splits);
 }

@@ -122,15 +122,17 @@ struct MatchedPlan {
   int64_t k_per_split;
   int64_t chunk_rows;  // decode kernel: rows per launch (<= 16)
   size_t ws;           // workspace bytes
+  int swap_ctas;       // of the masked product (Plan)
 };
 
 MatchedPlan matched_plan(int64_t M, int64_t K, int64_t N, int64_t order_rows, spl_path resolved) {
-  MatchedPlan mp{false, 0, 1, K, M, 0};
+  MatchedPlan mp{false, 0, 1, K, M, 0, 0};
   const Plan online = make_plan(order_rows, K, N, resolved);
   mp.kernel = online.kernel;
   if (online.kernel == kKernelTc) {
-    int variant = 0;  // the bank runs its own launch shape; only the K-split order carries over
-    if (!tc_uniform_shape(order_rows, K, N, resolved, &variant, &mp.splits)) return mp;
+    mp.splits = tc_uniform_splits(online);  // the bank runs its own launch shape; only the K-split order carries over
+    mp.swap_ctas = online.swap_ctas;
+    if (mp.splits == 0) return mp;
     mp.ws = kCounterBytes + tc_asplit_bytes(M, K, resolved) + tc_partial_bytes(M, K, N, order_rows, resolved);
     mp.ok = true;
     return mp;
@@ -352,7 +354,7 @@ spl_status precompute_matched(float* C, const float* Nz, const spl_weight* A, co
     args.a_l16 = A->f16_lo;
     args.a_exp = A->f16_exp;
   }
-  if (mp.kernel == kKernelTc) return run_tc_matched(args, order_rows);
+  if (mp.kernel == kKernelTc) return run_tc_matched(args, mp.splits, mp.swap_ctas);
   Plan p{};
   p.kernel = mp.kernel;
   p.splits = mp.splits;
