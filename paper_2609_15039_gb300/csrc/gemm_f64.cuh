@@ -16,7 +16,8 @@
 // So the only errors are the roundings to fixed point (2^-54 of the row's largest entry each), the dropped
 // products and the conversion of the result.  Against gamma_K S (S the sum of the terms' magnitudes) that
 // is small unless S is far below the rows' largest entries, which f64_finish_kernel checks for every output
-// (f64_guard_ok): an output that fails, or whose rows hold an infinity or NaN, is summed again in binary64.
+// (by samples of K, then by more of it): an output that fails, or whose rows hold an infinity or NaN, is summed again
+// in binary64, by the same kernel.
 //
 // Kernel: one CTA per 128 rows of W (the MMA's rows) x TN tokens (its columns) over a K range.  16 worker
 // warps load the fp32 / binary64 tiles (cp.async, a stage ahead, each thread its own groups of 4 entries),
@@ -123,6 +124,16 @@ __device__ __forceinline__ void tmem_wait_ld(uint32_t (&a)[4], uint32_t (&b)[4],
 
 // What the slices need of a row: its largest biased exponent field (at least 1; kRowNonFinite with an
 // infinity or NaN; 0 for a row of zeros) and the mean magnitude in units of 2^E.
+template <class TX>
+struct F64Pair;
+template <>
+struct F64Pair<float> {
+  using type = float2;
+};
+template <>
+struct F64Pair<double> {
+  using type = double2;
+};
 struct F64Row {
   int e;
   float mean;
@@ -462,17 +473,159 @@ __device__ __forceinline__ float relative(double v, int e) {
   return ex > 0 && (u >> 20) ? __uint_as_float(((uint32_t)ex << 23) | ((u & 0xFFFFFu) << 3)) : 0.f;
 }
 
+// Shared memory of a block of 32 x 32 outputs.
+constexpr int kSumRow = 33;
+struct F64Block {
+  alignas(16) float ws[32][kGuardK + 4], xs[32][kGuardK + 4];  // sampled entries; once read, ws holds sums
+  F64Row wr[32], xr[32];
+  uint32_t soft[32], hard[32], done[32];  // by row, a bit a column: not cleared by the samples; not finite; summed again
+  __device__ double* sums() { return reinterpret_cast<double*>(&ws[0][0]); }
+};
+static_assert(sizeof(double) * 32 * kSumRow <= sizeof(float) * 32 * (kGuardK + 4), "the block's sums");
+
+// The V values of each lane summed over the warp: a lane gets the total of value lane / (32 / V) (halves exchanged while
+// more than one is left: V - 1 sums and then log2(32 / V), not 5 V; in binary64 each costs 16 cycles of the SM's pipe).
+template <int V, class T>
+__device__ __forceinline__ T warp_totals(T (&v)[V], int lane) {
+  int o = 16;
+#pragma unroll
+  for (int c = V; c >= 2; c /= 2, o /= 2) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < c / 2; ++i) {
+      const T send = up ? v[i] : v[i + c / 2], keep = up ? v[i + c / 2] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+#pragma unroll
+  for (; o > 0; o /= 2) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+  return v[0];
+}
+// Cells of a 32 x 32 block that the sampled bound does not clear, R rows (mr, mr + 1, ...) by 4 columns (nc, ...) a warp:
+// those in `soft` (bit 4 r + c) are cleared when S over more of K, then all of it, does it; the others and those in
+// `hard` are summed in binary64, each lane 2 of K at a time.  Returns the cells summed, their sums in res.
+// The whole call, us, at 8192 by 3072 and 1, 16, 128 rows; last what the FP64 pipe's kernel (fp64.cu) takes of any rows:
+//   all cleared by the samples             104   107   247
+//   an entry a row 1000 times the others   109   142   401   (each summed again by a warp of its own: 692, 1985, 4660)
+//   10000 times                            126   644  4628   (700, 2197, 6992)
+//   an infinity in one row                 252   256   533   (1991, 2059, 2434)
+//   every output summed again              316  1924  9013   (1967, 7041, 19080)
+//   FP64 pipe                              129   958  7421
+// Bound there by the FP64 pipe of the SMs that hold the blocks (96 of them up to 32 rows); small outputs have few: 16 x
+// 512 by 512, an entry of 1000 a row, 69 us (117; 39 on the pipe).
+template <int R, class TX>
+__device__ __forceinline__ uint32_t f64_again(const float* __restrict__ W, const TX* __restrict__ X, int64_t M,
+                                              int64_t K, int64_t N, int64_t mr, int64_t nc, const F64Row* xr,
+                                              const F64Row* wr, uint32_t soft, uint32_t hard, float part, double* res) {
+  using X2 = typename F64Pair<TX>::type;
+  constexpr int V = 4 * R, LPV = 32 / V;  // cells, lanes a cell
+  constexpr int64_t kRun = 512;           // of K between two looks at S
+  const int lane = threadIdx.x & 31, cell = lane / LPV;
+  const int r_max = (int)std::min<int64_t>(R - 1, M - 1 - mr), c_max = (int)std::min<int64_t>(3, N - 1 - nc);
+  const float* w0 = W + nc * K + 2 * lane;
+  const TX* x0 = X + mr * K + 2 * lane;
+  if (soft != 0u) {
+    float S[V];
+#pragma unroll
+    for (int i = 0; i < V; ++i) S[i] = 0.f;
+    const float mean = wr[std::min(cell & 3, c_max)].mean + xr[std::min(cell >> 2, r_max)].mean;
+    for (int64_t k0 = 0; k0 < K && soft != 0u; k0 += kRun) {
+      const int64_t k1 = std::min(K, k0 + kRun) - 2 * lane;
+#pragma unroll(R == 1 ? 4 : 1)
+      for (int64_t k = k0; k < k1; k += 64) {
+        float2 w[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) w[c] = __ldg(reinterpret_cast<const float2*>(w0 + std::min(c, c_max) * K + k));
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const int e = max(wr[std::min(c, c_max)].e, 1);
+          w[c] = make_float2(relative(w[c].x, e), relative(w[c].y, e));
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const X2 x = __ldg(reinterpret_cast<const X2*>(x0 + std::min(r, r_max) * K + k));
+          const int e = max(xr[std::min(r, r_max)].e, 1);
+          const float xa = relative(x.x, e), xb = relative(x.y, e);
+#pragma unroll
+          for (int c = 0; c < 4; ++c) S[4 * r + c] = fmaf(w[c].x, xa, fmaf(w[c].y, xb, S[4 * r + c]));
+        }
+      }
+      float t[V];
+#pragma unroll
+      for (int i = 0; i < V; ++i) t[i] = S[i];
+      const bool clear = warp_totals<V>(t, lane) * part >= 0.51f * mean + 0.041f;
+      soft &= ~__reduce_or_sync(0xffffffffu, clear ? 1u << cell : 0u);
+    }
+  }
+  const uint32_t need = soft | hard;
+  if (need == 0u) return 0u;
+  double v[V];
+#pragma unroll
+  for (int i = 0; i < V; ++i) v[i] = 0.0;
+#pragma unroll(R == 1 ? 4 : 1)
+  for (int64_t k = 0; k < K - 2 * lane; k += 64) {
+    float2 w[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) w[c] = __ldg(reinterpret_cast<const float2*>(w0 + std::min(c, c_max) * K + k));
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const X2 x = __ldg(reinterpret_cast<const X2*>(x0 + std::min(r, r_max) * K + k));
+      const double xa = (double)x.x, xb = (double)x.y;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) v[4 * r + c] = fma(xb, (double)w[c].y, fma(xa, (double)w[c].x, v[4 * r + c]));
+    }
+  }
+  const double t = warp_totals<V>(v, lane);
+  if (lane % LPV == 0 && (need >> cell & 1u)) res[(cell >> 2) * kSumRow + (cell & 3)] = t;
+  return need;
+}
+
+// The block's flagged cells, 4 rows x 4 columns a task, tasks dealt out to the 8 warps.  Not inlined: the kernel's own
+// registers stay those of the common case.
 template <class TX>
-__global__ void __launch_bounds__(256) f64_finish_kernel(double* __restrict__ out64, float* __restrict__ out32,
+__device__ __noinline__ void f64_again_block(F64Block* blk, const float* __restrict__ W, const TX* __restrict__ X,
+                                             int64_t M, int64_t K, int64_t N, int64_t m0, int64_t n0, float part) {
+  double* res = blk->sums();
+  for (int t = threadIdx.x >> 5; t < 64; t += 8) {
+    const int g = 4 * (t >> 3), q = 4 * (t & 7);
+    uint32_t sb = 0u, hb = 0u;
+    int rows_in = 0, last = 0;
+    for (int r = 0; r < 4; ++r) {
+      const uint32_t a = blk->soft[g + r] >> q & 15u, b = blk->hard[g + r] >> q & 15u;
+      sb |= a << (4 * r);
+      hb |= b << (4 * r);
+      if (a | b) {
+        ++rows_in;
+        last = r;
+      }
+    }
+    if (rows_in == 0) continue;
+    uint32_t done;
+    if (rows_in == 1)
+      done = f64_again<1, TX>(W, X, M, K, N, m0 + g + last, n0 + q, blk->xr + g + last, blk->wr + q, sb >> (4 * last),
+                              hb >> (4 * last), part, res + (g + last) * kSumRow + q)
+             << (4 * last);
+    else
+      done = f64_again<4, TX>(W, X, M, K, N, m0 + g, n0 + q, blk->xr + g, blk->wr + q, sb, hb, part,
+                              res + g * kSumRow + q);
+    if ((threadIdx.x & 31) == 0)
+      for (int r = 0; r < 4; ++r) atomicOr(&blk->done[g + r], (done >> (4 * r) & 15u) << q);
+  }
+}
+
+template <class TX>
+__global__ void __launch_bounds__(256, 3) f64_finish_kernel(double* __restrict__ out64, float* __restrict__ out32,
                                                          const long long* __restrict__ hi,
                                                          const uint32_t* __restrict__ lo,
                                                          const F64Row* __restrict__ rows,
                                                          const float* __restrict__ W, const TX* __restrict__ X,
                                                          const double* __restrict__ c, int splits, int64_t M, int64_t K,
                                                          int64_t N, int mode) {
-  constexpr int P = kGuardK + 4;
-  __shared__ __align__(16) float ws[32][P], xs[32][P];
-  __shared__ F64Row wr[32], xr[32];
+  __shared__ F64Block blk;
+  auto& ws = blk.ws;
+  auto& xs = blk.xs;
+  auto& wr = blk.wr;
+  auto& xr = blk.xr;
   pdl_wait();
   pdl_trigger();
   const int64_t n0 = (int64_t)blockIdx.x * 32, m0 = (int64_t)blockIdx.y * 32;
@@ -529,35 +682,44 @@ __global__ void __launch_bounds__(256) f64_finish_kernel(double* __restrict__ ou
         l[i] += (long long)__ldcg(lo + o);
       }
     }
+  double out[4];
+  uint32_t flagged = 0u;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int64_t m = m0 + 4 * warp + i;
-    if (m >= M) break;  // the same for the whole warp
     const F64Row rx = xr[4 * warp + i];
-    double r = 0.0;
-    bool again = false;
-    if (n < N) {
+    bool soft = false, hard = false;
+    out[i] = 0.0;
+    if (m < M && n < N) {
       const long long top = h[i] + (l[i] >> 32), low = l[i] & 0xFFFFFFFFll;
       // value (top 2^32 + low) 2^(40 - 106 + E_w + E_x), E = e - 127 or e - 1023
       const int sc = 40 - 106 + (max(rw.e, 1) - 127) + (max(rx.e, 1) - (sizeof(TX) == 8 ? 1023 : 127));
       const int s1 = sc / 2, s2 = sc - s1;  // in two exact steps, each a normal power of two
-      r = fma((double)top, 4294967296.0, (double)low) * __hiloint2double((s1 + 1023) << 20, 0) *
-          __hiloint2double((s2 + 1023) << 20, 0);
+      out[i] = fma((double)top, 4294967296.0, (double)low) * __hiloint2double((s1 + 1023) << 20, 0) *
+               __hiloint2double((s2 + 1023) << 20, 0);
+      hard = rw.e == kRowNonFinite || rx.e == kRowNonFinite;
       const bool zero = rw.e == 0 || rx.e == 0;  // a row of zeros (with a finite one): exactly 0
-      const bool finite = rw.e != kRowNonFinite && rx.e != kRowNonFinite;
-      again = !finite || (!zero && !(S[i] * part >= 0.51f * (rw.mean + rx.mean) + 0.041f));
+      soft = !hard && !zero && !(S[i] * part >= 0.51f * (rw.mean + rx.mean) + 0.041f);
     }
-    for (uint32_t todo = __ballot_sync(0xffffffffu, again); todo; todo &= todo - 1) {  // binary64, as a warp
-      const int who = __ffs(todo) - 1;
-      const float* w = W + (n0 + who) * K;
-      const TX* x = X + m * K;
-      double v = 0.0;
-      for (int64_t k = lane; k < K; k += 32) v = fma((double)__ldg(x + k), (double)__ldg(w + k), v);
+    const uint32_t sm = __ballot_sync(0xffffffffu, soft), hm = __ballot_sync(0xffffffffu, hard);
+    if (lane == 0) {
+      blk.soft[4 * warp + i] = sm;
+      blk.hard[4 * warp + i] = hm;
+      blk.done[4 * warp + i] = 0u;
+    }
+    flagged |= sm | hm;
+  }
+  if (__syncthreads_or((int)flagged) != 0) {
+    f64_again_block<TX>(&blk, W, X, M, K, N, m0, n0, part);
+    __syncthreads();
 #pragma unroll
-      for (int q = 16; q > 0; q >>= 1) v += __shfl_xor_sync(0xffffffffu, v, q);
-      if (lane == who) r = v;
-    }
-    if (n < N) finish_f64(out64, out32, m * N + n, r, c, mode);
+    for (int i = 0; i < 4; ++i)
+      if (blk.done[4 * warp + i] >> lane & 1u) out[i] = blk.sums()[(4 * warp + i) * kSumRow + lane];
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int64_t m = m0 + 4 * warp + i;
+    if (m < M && n < N) finish_f64(out64, out32, m * N + n, out[i], c, mode);
   }
 }
 
