@@ -23,8 +23,9 @@
 // split keeps fp32's exponent range) or FP32.  W is split once, offline; A is split by a pass before the product
 // into the workspace, so TMA lands every operand tile directly.
 //
-// FP16X3 products from about 256 rows on run on SM pairs (gemm_pair.cuh), those of 9 to 16 rows on the swapped
-// kernel (below).  The others: one CTA per 128 x BN output tile, 6 warps; BN = 128 to 256 with a ring of 192 or
+// FP16X3 products of 9 to 16 rows run on the swapped kernel (below), others on SM pairs (gemm_pair.cuh) where the
+// launch model finds them faster: most products of several hundred rows, and wide ones of fewer (from 17 rows on).
+// The rest: one CTA per 128 x BN output tile, 6 warps; BN = 128 to 256 with a ring of 192 or
 // 224 KB and one CTA per SM, or (TF32X3) BN = 128 with 96 KB and two, one's epilogue beside the other's mainloop:
 //   warp 0      TMA producer: per stage A_hi, A_lo, W_hi, W_lo.
 //   warp 1      TMEM allocator and MMA issuer: per stage 3 products per k-step into one
@@ -1576,7 +1577,8 @@ int swap_width_index(int64_t tokens) {
 // and Qwen projections at 24 to 2048 rows, and 150 drawn shapes of 17 to 2048 rows, K 64 to 9728 and N to 32768, many
 // of no round size.  The picks are within 0.2 to 0.4% of the best form measured on average over the projections
 // (4.4% at worst) and within 1.7% over the drawn shapes (23%, at 45 us); constants fitted to the projections alone
-// were 8.8% off there and 78% at worst, with pairs for short K and ragged N.  F32 and b32 are
+// were 8.8% off there and 78% at worst, with pairs for short K and ragged N.  (The limit on a form's error, below, and
+// the folds of unsplit tiles add 0.6% on average over 1500 drawn shapes and 7% at most, by the model.)  F32 and b32 are
 // TF32X3's, in elements of K of a 256-wide tile, fitted to the projections at 128 to 4096 rows (with FP16X3's constants
 // 200 by 1708 by 5000 took 45.8 us instead of 41.7).
 struct Variant {
@@ -1584,8 +1586,9 @@ struct Variant {
   double F, b, F32, b32;
 };
 constexpr int kVariants = 6;
+constexpr double kNever = 1e9;  // FP16X3 with two CTAs per SM: only the test hook launches it (tc_shape_for says why)
 constexpr Variant kVariant[kVariants] = {{256, 192, 1, 8.03, 15.01, 500.0, 1.00}, {128, 224, 1, 5.66, 9.76, 300.0, 1.05},
-                                         {128, 96, 2, 0.0, 0.0, 250.0, 0.95},     {160, 224, 1, 5.66, 11.62, 250.0, 1.05},
+                                         {128, 96, 2, kNever, kNever, 250.0, 0.95},     {160, 224, 1, 5.66, 11.62, 250.0, 1.05},
                                          {192, 224, 1, 7.10, 11.62, 300.0, 1.00}, {224, 224, 1, 6.21, 15.41, 550.0, 0.97}};
 
 // Co-resident clusters of s CTAs of variant v on the current device; clusters must fit inside
@@ -1612,10 +1615,15 @@ int query_active_clusters(int s) {
   return n;
 }
 
-int max_active_clusters(int v, int s, int sms) {
-  static int cache[64][kVariants][MAX_CLUSTER + 1] = {{{0}}};
+// The current device, below 64; -1 without one.  A plan asks once for its hundred or so occupancy look-ups.
+int current_device() {
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return std::max(1, sms * kVariant[v].cps / s);
+  return cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 ? dev : -1;
+}
+
+int max_active_clusters(int v, int s, int sms, int dev) {
+  static int cache[64][kVariants][MAX_CLUSTER + 1] = {{{0}}};
+  if (dev < 0) return std::max(1, sms * kVariant[v].cps / s);
   int& c = cache[dev][v][s];
   if (c == 0) {
     int n = 0;
@@ -1634,7 +1642,7 @@ int max_active_clusters(int v, int s, int sms) {
 
 // Widths of the pair kernel's 256-row tiles (FP16X3) and their cost in us: F once, then per tile of the
 // busiest pair b K plus h (the part of a tile's hand-over and epilogue that its successor does not hide).
-// Fitted with the variants above.  A pair beats two single SMs from about 256 rows on: its tile needs
+// Fitted with the variants above.  A pair beats two single SMs once its 256 rows are about filled: its tile needs
 // 32 KB a k-block per SM where a 128 x 256 tile needs 48, so the tensor pipe is not kept waiting
 // (256-wide: 11.7 against 15.0 us per 1000 of K).  Times at 1024 rows (with the split of A): 3072 by 16384
 // 229 -> 179 us, 3072 by 3072 48 -> 44 us, 8192 by 3072 122 -> 101 us; at 4096 rows 3072 by 16384
@@ -1653,10 +1661,9 @@ constexpr int kPairRingKb = 448;  // how the test hooks name the pair variants: 
 
 // Co-resident pairs of the pair kernel (clusters of two CTAs, one CTA per SM).
 template <int BN>
-int active_pairs() {
+int active_pairs(int dev) {
   static int cache[64] = {0};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return std::max(1, device_sm_count() / 2);
+  if (dev < 0) return std::max(1, device_sm_count() / 2);
   if (cache[dev] == 0) {
     int n = 0;
     cudaLaunchConfig_t cfg;
@@ -1680,13 +1687,13 @@ int active_pairs() {
   return cache[dev];
 }
 
-int pairs_of(int w) {
+int pairs_of(int w, int dev) {
   switch (w) {
-    case 0: return active_pairs<kPair[0].bn>();
-    case 1: return active_pairs<kPair[1].bn>();
-    case 2: return active_pairs<kPair[2].bn>();
-    case 3: return active_pairs<kPair[3].bn>();
-    default: return active_pairs<kPair[4].bn>();
+    case 0: return active_pairs<kPair[0].bn>(dev);
+    case 1: return active_pairs<kPair[1].bn>(dev);
+    case 2: return active_pairs<kPair[2].bn>(dev);
+    case 3: return active_pairs<kPair[3].bn>(dev);
+    default: return active_pairs<kPair[4].bn>(dev);
   }
 }
 
@@ -1698,6 +1705,7 @@ struct Problem {
   int64_t M, K, N;
   int sms;
   bool f16;
+  int dev = current_device();
   double k_us(double b, double straddle) const { return b * 1e-3 * (double)K * (K % 64 != 0 ? straddle : 1.0); }
   double ragged_us(double per_tile, int bn) const { return (N & 3) != 0 ? per_tile * bn / 128.0 : 0.0; }
   double fixed_us(double F, double part, int s) const {
@@ -1721,7 +1729,7 @@ constexpr double kPersistentTile = 6.73, kPersistentTile32 = 60.0;
 
 double launch_cost(const Problem& p, int v, int64_t tiles, int s) {
   if (tiles <= 0) return 0.0;
-  int64_t clusters = max_active_clusters(v, s, p.sms);
+  int64_t clusters = max_active_clusters(v, s, p.sms, p.dev);
   const Variant& w = kVariant[v];
   if (!p.f16) return (double)ceil_div(tiles, clusters) * (w.F32 + 20.0 * s + w.b32 * (double)p.K / (double)s);
   // clusters of 3, 5 or 7 CTAs: one fewer fits than the occupancy query says (exactly full grids of them
@@ -1785,7 +1793,7 @@ TcShape tc_shape_for(const Problem& p, int v, double max_error2) {
   TcShape best{v, 0, tiles, 1, 1e300};
   // FP16X3 of two CTAs per SM: never more than 4% faster than the other widths, 1.6% slower on average
   if (p.f16 && kVariant[v].cps > 1) return best;
-  const int64_t wave = max_active_clusters(v, 1, p.sms);
+  const int64_t wave = max_active_clusters(v, 1, p.sms, p.dev);
   for (int s = 1; s <= max_s; ++s) {
     if (p.f16 && s > 1 && (s - 1) * round_up(ceil_div(p.K, s), 32) >= p.K) continue;  // a rank without K
     if (p.f16 && (s == 1 ? unsplit_error2(p.K) : error2(p.K, s, 32 * kChainBlocks)) > max_error2) continue;
@@ -1822,7 +1830,7 @@ TcShape tc_shape_for(const Problem& p, int v, double max_error2) {
 
 double pair_cost(const Problem& p, int w) {
   const int64_t tiles = ceil_div(p.M, (int64_t)256) * ceil_div(p.N, (int64_t)kPair[w].bn);
-  return p.fixed_us(kPair[w].F, kShortPair, 1) + (double)ceil_div(tiles, (int64_t)pairs_of(w)) *
+  return p.fixed_us(kPair[w].F, kShortPair, 1) + (double)ceil_div(tiles, (int64_t)pairs_of(w, p.dev)) *
                           (p.k_us(kPair[w].b, kStraddlePair) + kPair[w].h + p.ragged_us(kRaggedPair, kPair[w].bn) +
                            kFoldPair * more_folds(p.K));
 }
@@ -1852,7 +1860,7 @@ TcShape tc_bank_shape(int64_t M, int64_t K, int64_t N, int seg_splits, int sms, 
     const double c = launch_cost(p, v, tiles, 1);
     if (c < best.cost * (1.0 - 1e-9)) best = TcShape{v, 0, tiles, 1, c};
     if (seg_splits < 2 || seg_splits > MAX_CLUSTER) continue;
-    const int64_t wave = max_active_clusters(v, 1, sms);
+    const int64_t wave = max_active_clusters(v, 1, sms, p.dev);
     const int64_t full = (tiles / wave) * wave, rest = tiles - full;
     if (rest == 0) continue;
     const double c2 = launch_cost(p, v, full, 1) + (f16 && full > 0 ? kRound : 0.0) + launch_cost(p, v, rest, seg_splits);
@@ -1936,7 +1944,7 @@ spl_status launch_tc(const LinearArgs& a, const uint16_t* a_hi, const uint16_t* 
     if (!set_smem_attr_persistent<Md, BN, RK>()) return SPL_ECUDA;
     const int64_t tiles = shape.full_tiles + shape.rest_tiles;
     if (tiles > 0x7fffffffLL) return SPL_ESHAPE;
-    const int ctas = (int)std::min<int64_t>(tiles, max_active_clusters(shape.v, 1, device_sm_count()));
+    const int ctas = (int)std::min<int64_t>(tiles, max_active_clusters(shape.v, 1, device_sm_count(), current_device()));
     cudaLaunchConfig_t cfg;
     std::memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3((unsigned)ctas, 1, 1);
@@ -2010,7 +2018,7 @@ spl_status launch_pair_bn(const LinearArgs& a, const uint16_t* a_hi, const uint1
       (tma_epi && !make_map(&maps.y, a.out, false, a.M, a.N, 32, 32, CU_TENSOR_MAP_SWIZZLE_128B)) ||
       (tma_epi && c_rows > 0 && !make_map(&maps.c, a.c, false, c_rows, a.N, 32, 32, CU_TENSOR_MAP_SWIZZLE_128B)))
     return SPL_ECUDA;
-  const int64_t pairs = std::min<int64_t>(tiles, active_pairs<BN>());
+  const int64_t pairs = std::min<int64_t>(tiles, active_pairs<BN>(current_device()));
   cudaLaunchConfig_t cfg;
   std::memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3((unsigned)(2 * pairs), 1, 1);
@@ -2355,12 +2363,12 @@ extern "C" spl_status spl_test_tc_capacity(int64_t tile_n, int64_t ring_kb, int6
   if (!out || cluster < 1 || cluster > MAX_CLUSTER) return SPL_EINVAL;
   for (int v = 0; v < kVariants; ++v)
     if (kVariant[v].bn == tile_n && kVariant[v].rk == ring_kb) {
-      *out = max_active_clusters(v, (int)cluster, device_sm_count());
+      *out = max_active_clusters(v, (int)cluster, device_sm_count(), current_device());
       return SPL_OK;
     }
   for (int w = 0; w < kPairs; ++w)
     if (kPair[w].bn == tile_n && ring_kb == kPairRingKb && cluster <= 2) {
-      *out = (int64_t)pairs_of(w) * (cluster == 1 ? 2 : 1);
+      *out = (int64_t)pairs_of(w, current_device()) * (cluster == 1 ? 2 : 1);
       return SPL_OK;
     }
   return SPL_EINVAL;
