@@ -280,10 +280,10 @@ spl_status spl_masked_linear_unmask(float* Y, const float* Xt, const spl_weight*
  *   spl_masked_linear_unmask_f64: Y = fl32(fl64(Xt W^T) - C), Xt and C binary64,
  *                         W fp32, products rounded once in binary64, binary64 sums.
  * The sums are binary64 ones (gamma_K with u = 2^-53 bounds their error): added in
- * binary64 on the FP64 pipe, or, from a few rows on, of exact products of slices
- * of the operands on the tensor cores (every output whose terms the slices might
- * not hold to that bound, and rows with an infinity or NaN, are summed again in
- * binary64).  Workspace: spl_f64_workspace_bytes(M, K, N) (the
+ * binary64 on the FP64 pipe, or, for all but small products, of exact products of
+ * slices of the operands on the tensor cores (every output whose terms the slices
+ * might not hold to that bound, and rows with an infinity or NaN, are summed again
+ * in binary64).  Workspace: spl_f64_workspace_bytes(M, K, N) (the
  * first 64 KiB are left untouched, so the product workspace can be shared).
  * Errors as spl_masked_linear (all base pointers 16-byte aligned, K % 4 == 0). */
 spl_status spl_noise_mask_f64(double* Xt, const float* X, int64_t rows, int64_t cols, double sensitivity,

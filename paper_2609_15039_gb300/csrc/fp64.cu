@@ -7,9 +7,9 @@
 // binary64, the correction W eta is kept in binary64 and subtracted in binary64; only Y is rounded
 // to fp32 at the end.
 //
-// Products of a few rows on run as exact slices on the tensor cores (gemm_f64.cuh, by the rule in fp64.cuh),
-// whose result is closer to the exact sum than a binary64 sum's.  The kernels here take the rest, on the FP64
-// pipe.
+// All but small products run as exact slices on the tensor cores (gemm_f64.cuh, by the rule in fp64.cuh), whose
+// result is closer to the exact sum than a binary64 sum's.  The kernels here take the rest, and calls whose workspace
+// is too small for the slices, on the FP64 pipe.
 //
 // Kernel: the decode kernel's structure in binary64 -- a 256-thread block owns 16 rows of W over
 // a K-slice, stages MT (1, 2, 4 or 8) rows of the left operand of that slice in shared memory (as

@@ -38,7 +38,11 @@ __device__ __forceinline__ void finish_f64(double* out64, float* out32, int64_t 
 // 248 us (5.2 ms at the pipe's rate), 16 rows 946 against 95, 1 row 118 against 88; 16 x 512 by 512 26 against 18,
 // 4 x 1024 by 1024 27 against 20, but 8 x 512 by 512 15 against 18; of one row 4096 by 2048 43 against 37 and
 // 2048 by 2048 25 against 27, and with short rows 512 by 16384 41 against 54.  The bounds on K and the sizes keep
-// the 96-bit sums and the grids in range.
+// the 96-bit sums and the grids in range.  Those are times of rows that the slices hold; what others cost stands at
+// f64_again.
+// Slalom's integers (below 2^24, sums below 2^53) lose nothing in the slices: in fixed point below the row's largest
+// exponent E <= 23 an integer is a multiple of 2^30, so its digits 0, 1 and 2 are 0, every product of two digits that
+// are not (p + s >= 6) is kept, and the exact sum, of at most 53 bits, becomes a double without rounding.
 inline bool f64_on_tensor_cores(int64_t M, int64_t K, int64_t N) {
   if (K >= (int64_t(1) << 21) || M >= (int64_t(1) << 19) || N >= (int64_t(1) << 20)) return false;
   if (M < 4) return K >= 2048 && K * N >= (int64_t(1) << 23);

@@ -205,6 +205,21 @@ def test_slices_pass_infinities_and_nans_on(spl):
     assert torch.equal(got[keep], clean[keep])
 
 
+@pytest.mark.parametrize("top_x,top_w", [(24, 8), (23, 24), (1, 1), (12, 16)])
+def test_slices_of_integers_are_exact(spl, top_x, top_w):
+    """Slalom's products: integers below 2^24 whose sums stay below 2^53 lose nothing in the slices."""
+    M, K, N = 37, 1028, 514
+    g = torch.Generator(device="cuda").manual_seed(top_x)
+    K_cut = K if top_x + top_w + 11 <= 53 else 60  # 60 terms of 2^47: the rest of the row is 0
+    X = torch.randint(-2 ** top_x + 1, 2 ** top_x, (M, K), generator=g, device="cuda")
+    W = torch.randint(-2 ** top_w + 1, 2 ** top_w, (N, K), generator=g, device="cuda")
+    X[:, K_cut:] = 0
+    X[:, 0] = 1 - 2 ** top_x
+    got = _product(spl, X.float(), W.float()).cpu()
+    want = (X.cpu() @ W.cpu().T).double()
+    assert torch.equal(got, want)
+
+
 @pytest.mark.parametrize("seed", [1, 2])
 def test_slices_are_closer_than_a_binary64_sum(spl, seed):
     """No less precise than the FP64 pipe: over noise-like rows of the Down shape the error of the slices, in units
