@@ -138,6 +138,7 @@ struct TcShape {
   double cost;              // shape_rank (us on FP16X3)
   bool persistent = false;  // one launch of tc_persistent_kernel over every tile (unsplit)
   int pair = -1;            // >= 0: width index of tc_pair_kernel, one launch over every tile (unsplit)
+  int chain = 32;           // k-blocks per accumulation chain of unsplit tiles (at most kChainBlocks)
 };
 
 // Split-K plans: how many K-splits each kernel uses and the workspace it needs.
@@ -181,9 +182,9 @@ int64_t gemv_max_ks(int64_t M);                           // largest K-slice the
 // K-split of a planned tcgen05 call of one launch (1 for the swapped kernel of few rows); 0 if it makes two.
 int tc_uniform_splits(const Plan& p);
 // A tcgen05 product whose every output is summed in the order of the masked product that was planned with
-// tc_uniform_splits `splits` and `swap_ctas` (the correction bank): the same K ranges, accumulation chains and
+// tc_uniform_splits `splits`, `swap_ctas` and, where K is not split, chains of `chain` k-blocks (the correction bank): the same K ranges, accumulation chains and
 // cluster order.
-spl_status run_tc_matched(const LinearArgs& a, int splits, int swap_ctas);
+spl_status run_tc_matched(const LinearArgs& a, int splits, int swap_ctas, int chain);
 size_t tc_asplit_bytes(int64_t M, int64_t K, spl_path path);  // FP16X3 split of A in the workspace (0 for TF32X3)
 // Workspace for the partial tiles of a tcgen05 product of M rows summed in the order of `order_rows`
 // (the swapped kernel's runs; 0 for the cluster-reduced kernels), after the split of A.

@@ -78,16 +78,13 @@ constexpr int MAX_CLUSTER = 8;                         // split-K CTAs of one ou
 // the running sum with a round-to-nearest fp32 add (R = fl(R + P)), so the bias of every chain is
 // bounded whatever K is, and the folds' own errors are unbiased.  A fold costs ~0.35 us per CTA.
 constexpr int kChainBlocks = 32;
-// FP16X3 tiles whose K is not split: chains of 512 elements.  The error of a correction then halves (at K = 3072
-// 3.6e-6 -> 1.8e-6 of the result's norm, against 64 bits; a K-split over 3, 4, 5 or 6 CTAs has 3.6, 2.7, 2.2 and
-// 1.8e-6), and on pairs, which fold in registers beside the MMAs, it costs at most 1%: 1024 x 3072 by 16384 175.2 ->
-// 175.7 us, by 5120 67.0 -> 67.8 (chains of 256: 181.3 and 71.9).  Single SMs fold in TMEM while the MMAs wait: 61 x
-// 2560 by 19456, which HBM bounds, 39.5 -> 39.7 us; 128 x 3072 by 5120 unsplit 38.8 -> 40.0.
-constexpr int kUnsplitBlocks = 16;
-template <class Md>
-constexpr int chain_blocks(int splits) {  // longest chain of a CTA whose K is split `splits` ways
-  return Md::kF16 && splits == 1 ? kUnsplitBlocks : kChainBlocks;
-}
+// FP16X3 tiles whose K is not split take chains of 512 elements where 1024 would round more than the launch model
+// allows (error2_limit).  The error of a correction then halves (at K = 3072 3.6e-6 -> 1.8e-6 of the result's norm,
+// against 64 bits; a K-split over 3, 4, 5 or 6 CTAs has 3.6, 2.7, 2.2 and 1.8e-6).  On pairs, which fold in registers
+// beside the MMAs, it costs about 1%: 1024 x 3072 by 16384 175.2 -> 175.7 us, by 5120 67.0 -> 67.8 (chains of 256: 181.3
+// and 71.9), the 28-layer prefill step 12.03 -> 12.34 ms with 512 everywhere.  Single SMs fold in TMEM while the MMAs
+// wait: 61 x 2560 by 19456, which HBM bounds, 39.5 -> 39.7 us; 128 x 3072 by 5120 unsplit 38.8 -> 40.0.
+constexpr int kShortBlocks = 16;
 constexpr uint32_t AUX_BYTES = 2048;                   // barriers, TMEM slot, abort flag; column scales at +1024
 
 // ---- instruction descriptors (tcgen05.mma kind::tf32 / kind::f16) ---------------
@@ -1706,6 +1703,7 @@ struct Problem {
   int sms;
   bool f16;
   int dev = current_device();
+  int chain = kChainBlocks;  // k-blocks per chain of unsplit tiles
   double k_us(double b, double straddle) const { return b * 1e-3 * (double)K * (K % 64 != 0 ? straddle : 1.0); }
   double ragged_us(double per_tile, int bn) const { return (N & 3) != 0 ? per_tile * bn / 128.0 : 0.0; }
   double fixed_us(double F, double part, int s) const {
@@ -1719,9 +1717,9 @@ constexpr double kRound = 4.0;                            // each further round:
 // Folds beyond those of chains of kChainBlocks (with which the constants were fitted), us each and round: in TMEM, in
 // TMEM beside the next tile's MMAs, in registers beside them.
 constexpr double kFold = 0.35, kFoldPersistent = 0.8, kFoldPair = 0.13;
-int more_folds(int64_t K) {
+int more_folds(int64_t K, int chain) {
   const int64_t nkb = ceil_div(K, (int64_t)32);
-  return (int)(ceil_div(nkb, (int64_t)kUnsplitBlocks) - ceil_div(nkb, (int64_t)kChainBlocks));
+  return (int)(ceil_div(nkb, (int64_t)chain) - ceil_div(nkb, (int64_t)kChainBlocks));
 }
 // The single-SM persistent form: F once, then per tile of the busiest CTA its mainloop and a hand-over.  It is left
 // where a 256-row tile would be half empty (up to 128 rows of several waves) and for TF32X3.
@@ -1738,7 +1736,7 @@ double launch_cost(const Problem& p, int v, int64_t tiles, int s) {
   const double rounds = (double)ceil_div(tiles, clusters);
   const double rows = (double)std::min<int64_t>(p.M, BM) / BM;
   return (rounds - 1.0) * kRound +
-         rounds * (p.fixed_us(w.F, kShort, s) + p.k_us(w.b, kStraddle) / (double)s + (s == 1 ? kFold * more_folds(p.K) : 0.0) +
+         rounds * (p.fixed_us(w.F, kShort, s) + p.k_us(w.b, kStraddle) / (double)s + (s == 1 ? kFold * more_folds(p.K, p.chain) : 0.0) +
                    p.ragged_us(kRagged * rows / s, w.bn) + (s > 1 && (p.N & 3) != 0 ? 1.0 : 0.0));
 }
 
@@ -1748,7 +1746,7 @@ double launch_cost(const Problem& p, int v, int64_t tiles, int s) {
 double shape_rank(const Problem& p, double cost, int splits) {
   if (!p.f16) return cost;
   const double bytes = 4.0 * (double)(p.N + p.M) * (double)p.K + 8.0 * (double)p.M * (double)p.N;
-  const int64_t longest = 32 * chain_blocks<Fp16x3>(splits);
+  const int64_t longest = 32 * (splits == 1 ? p.chain : kChainBlocks);
   const double chain = (double)std::min<int64_t>(longest, round_up(ceil_div(p.K, splits), 32));
   return std::max(cost, 5.1 + bytes / 6.7e6) + 0.1 * splits + 0.12 * chain / 256.0;
 }
@@ -1782,7 +1780,7 @@ double error2_limit(const Problem& p) {
   return (full * error2(p.K, 1, 32 * kChainBlocks) + rest * error2(p.K, t.rest_splits, 32 * kChainBlocks)) / (full + rest) *
          (1.0 + 1e-9);
 }
-double unsplit_error2(int64_t K) { return error2(K, 1, 32 * kUnsplitBlocks); }
+double unsplit_error2(const Problem& p) { return error2(p.K, 1, 32 * p.chain); }
 
 TcShape tc_shape_for(const Problem& p, int v, double max_error2) {
   // the persistent epilogue stores whole float4s: output rows of whole 16-byte units (a launch whose
@@ -1796,7 +1794,7 @@ TcShape tc_shape_for(const Problem& p, int v, double max_error2) {
   const int64_t wave = max_active_clusters(v, 1, p.sms, p.dev);
   for (int s = 1; s <= max_s; ++s) {
     if (p.f16 && s > 1 && (s - 1) * round_up(ceil_div(p.K, s), 32) >= p.K) continue;  // a rank without K
-    if (p.f16 && (s == 1 ? unsplit_error2(p.K) : error2(p.K, s, 32 * kChainBlocks)) > max_error2) continue;
+    if (p.f16 && (s == 1 ? unsplit_error2(p) : error2(p.K, s, 32 * kChainBlocks)) > max_error2) continue;
     const double c = shape_rank(p, launch_cost(p, v, tiles, s), s);
     if (c < best.cost * (1.0 - 1e-9)) best = TcShape{v, 0, tiles, s, c};
   }
@@ -1814,11 +1812,11 @@ TcShape tc_shape_for(const Problem& p, int v, double max_error2) {
     }
   }
   if (persistent_ok && kVariant[v].cps == 1 && tiles > wave &&  // more than one wave of unsplit tiles
-      (!p.f16 || unsplit_error2(p.K) <= max_error2)) {
+      (!p.f16 || unsplit_error2(p) <= max_error2)) {
     const Variant& w = kVariant[v];
     const double rounds = (double)ceil_div(tiles, wave);
     const double c = shape_rank(p, p.f16 ? p.fixed_us(w.F, kShort, 1) + rounds * (p.k_us(w.b, kStraddle) + kPersistentTile +
-                                                                                         kFoldPersistent * more_folds(p.K))
+                                                                                         kFoldPersistent * more_folds(p.K, p.chain))
                                          : w.F32 + rounds * (w.b32 * (double)p.K + kPersistentTile32), 1);
     if (c < best.cost * (1.0 - 1e-9)) {
       best = TcShape{v, 0, tiles, 1, c};
@@ -1832,7 +1830,7 @@ double pair_cost(const Problem& p, int w) {
   const int64_t tiles = ceil_div(p.M, (int64_t)256) * ceil_div(p.N, (int64_t)kPair[w].bn);
   return p.fixed_us(kPair[w].F, kShortPair, 1) + (double)ceil_div(tiles, (int64_t)pairs_of(w, p.dev)) *
                           (p.k_us(kPair[w].b, kStraddlePair) + kPair[w].h + p.ragged_us(kRaggedPair, kPair[w].bn) +
-                           kFoldPair * more_folds(p.K));
+                           kFoldPair * more_folds(p.K, p.chain));
 }
 // The pair form of width w (FP16X3), every tile unsplit.  rest_tiles counts 128-row tiles, as the other forms do.
 TcShape pair_shape(const Problem& p, int w, double cost) {
@@ -1851,8 +1849,9 @@ int rank_blocks_of(int64_t K, int s) {
 // waves of unsplit tiles that fold the K ranges in TMEM (segmented mode), then the remaining
 // tiles with K split seg_splits ways over a cluster, whose rank-order sum is the same fold; or
 // every tile segmented, on single SMs or on pairs.  The cheapest variant and form.
-TcShape tc_bank_shape(int64_t M, int64_t K, int64_t N, int seg_splits, int sms, bool f16) {
-  const Problem p{M, K, N, sms, f16};
+TcShape tc_bank_shape(int64_t M, int64_t K, int64_t N, int seg_splits, int sms, bool f16, int chain) {
+  Problem p{M, K, N, sms, f16};
+  if (seg_splits == 1) p.chain = chain;
   TcShape best{0, 0, 0, 1, 1e300};
   for (int v = 0; v < kVariants; ++v) {
     if (f16 && kVariant[v].cps > 1) continue;
@@ -1870,45 +1869,46 @@ TcShape tc_bank_shape(int64_t M, int64_t K, int64_t N, int seg_splits, int sms, 
   if (f16 && (seg_splits == 1 || rank_blocks_of<Fp16x3>(K, seg_splits) <= kChainBlocks))
     for (int w = 0; w < kPairs; ++w)
       if (const double c = pair_cost(p, w); c < best.cost * (1.0 - 1e-9)) best = pair_shape(p, w, c);
+  best.chain = p.chain;
   return best;
 }
 
 TcShape tc_shape(int64_t M, int64_t K, int64_t N, int sms, bool f16) {
-  const Problem p{M, K, N, sms, f16};
+  Problem p{M, K, N, sms, f16};
   double limit = f16 ? error2_limit(p) : 1e300;
+  if (unsplit_error2(p) > limit) p.chain = kShortBlocks;
   for (;;) {
     TcShape best = tc_shape_for(p, 0, limit);
     for (int v = 1; v < kVariants; ++v) {
       const TcShape t = tc_shape_for(p, v, limit);
       if (t.cost < best.cost * (1.0 - 1e-9)) best = t;
     }
-    for (int w = 0; f16 && unsplit_error2(K) <= limit && w < kPairs; ++w)
+    for (int w = 0; f16 && unsplit_error2(p) <= limit && w < kPairs; ++w)
       if (const double c = shape_rank(p, pair_cost(p, w), 1); c < best.cost * (1.0 - 1e-9)) best = pair_shape(p, w, c);
+    best.chain = p.chain;
     if (best.cost < 1e299) return best;
     limit = 1e300;  // not met: the limit's own form is among those above or rounds more than the unsplit one
   }
 }
 
-// Segments of a CTA whose K range, one of `splits`, is k_range elements: chain_blocks when it is longer, else 0
-// (one chain).
+// Segments of a CTA whose K range is k_range elements: `chain` k-blocks when it is longer, else 0 (one chain).
 template <class Md>
-int chain_segments(int64_t k_range, int splits) {
-  const int chain = chain_blocks<Md>(splits);
+int chain_segments(int64_t k_range, int chain) {
   return ceil_div(k_range, (int64_t)Md::BK) > chain ? chain : 0;
 }
 
 template <class Md, int BN, int RK>
 spl_status launch_tc(const LinearArgs& a, const uint16_t* a_hi, const uint16_t* a_lo, const int* a_exp,
                      TcShape shape, int skip_kblock, int seg_splits) {
-  // Every CTA cuts its K range into chains of at most chain_blocks k-blocks.  A correction in the
+  // Every CTA cuts its K range into chains: of shape.chain k-blocks where K is not split, else of kChainBlocks.  A correction in the
   // order of a seg_splits-way split (seg_splits > 0, the bank) reproduces, per tile, what the online
   // product did: an online split of at most kChainBlocks k-blocks per rank is one chain per rank,
   // summed in rank order, which one CTA over all of K reproduces by folding segments cut at the
-  // split's boundaries; an unsplit online product (seg_splits = 1) is folded at chain_blocks(1); an
+  // split's boundaries; an unsplit online product (seg_splits = 1) is folded at its chains; an
   // online split whose ranks fold chains of their own is reproduced by the same cluster split.
   int seg_blocks = 0;  // segments of the unsplit tiles of a seg_splits launch
   if (seg_splits == 1) {
-    seg_blocks = chain_segments<Md>(a.K, 1);
+    seg_blocks = chain_segments<Md>(a.K, shape.chain);
   } else if (seg_splits > 1) {
     const int rank_blocks = rank_blocks_of<Md>(a.K, seg_splits);
     if (rank_blocks <= kChainBlocks) {
@@ -1958,7 +1958,7 @@ spl_status launch_tc(const LinearArgs& a, const uint16_t* a_hi, const uint16_t* 
     cfg.numAttrs = 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, tc_persistent_kernel<Md, BN, RK>, maps, a.out, a.c, a_exp,
                                              (const int*)a.w_exp, a.M, a.K, a.N, (int)tiles, m_tiles,
-                                             chain_blocks<Md>(1), a.c_rows);
+                                             shape.chain, a.c_rows);
     note_launches(1);
     return e == cudaSuccess ? SPL_OK : SPL_ECUDA;
   }
@@ -1969,7 +1969,7 @@ spl_status launch_tc(const LinearArgs& a, const uint16_t* a_hi, const uint16_t* 
   auto launch = [&](int64_t tiles, int64_t base, int splits, int seg) -> spl_status {
     if (tiles <= 0) return SPL_OK;
     const int64_t kps = round_up(ceil_div(a.K, splits), Md::BK);
-    if (seg == 0) seg = chain_segments<Md>(kps, splits);
+    if (seg == 0) seg = chain_segments<Md>(kps, splits == 1 ? shape.chain : kChainBlocks);
     cudaLaunchConfig_t cfg;
     std::memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3((unsigned)tiles, 1, (unsigned)splits);
@@ -2160,10 +2160,11 @@ spl_status launch_swap(const LinearArgs& a, const uint16_t* x_hi, const uint16_t
 // (0: the library's count, which depends on K and N only, so a bank of any width meets the online
 // product's runs).
 // pair_w >= 0: every tile on the pair kernel of that width index (FP16X3).
-// planned: the launch shape, where the caller has it (else it is worked out here).
+// planned: the launch shape, where the caller has it (else it is worked out here).  seg_chain: chain of the unsplit
+// product that seg_splits = 1 follows.
 spl_status run_tc_impl(const LinearArgs& a, int skip_kblock, int forced_v, int forced_splits, int seg_splits = 0,
                        int64_t forced_full = 0, bool forced_persistent = false, int swap_w = -1, int swap_s = 0,
-                       int pair_w = -1, const TcShape* planned = nullptr) {
+                       int pair_w = -1, const TcShape* planned = nullptr, int seg_chain = kChainBlocks) {
   const int cc = device_cc();
   if (cc != 100 && cc != 103) return SPL_EUNSUPPORTED;
   const bool f16 = a.path == SPL_PATH_FP16X3;
@@ -2225,7 +2226,7 @@ spl_status run_tc_impl(const LinearArgs& a, int skip_kblock, int forced_v, int f
     shape = TcShape{forced_v, forced_full, tiles - forced_full, forced_splits, 0.0};
     shape.persistent = forced_persistent;
   } else if (seg_splits > 0) {
-    shape = tc_bank_shape(a.M, a.K, a.N, seg_splits, device_sm_count(), f16);
+    shape = tc_bank_shape(a.M, a.K, a.N, seg_splits, device_sm_count(), f16, seg_chain);
   } else {
     shape = planned ? *planned : tc_shape(a.M, a.K, a.N, device_sm_count(), f16);
   }
@@ -2234,7 +2235,7 @@ spl_status run_tc_impl(const LinearArgs& a, int skip_kblock, int forced_v, int f
   const uint16_t* lo = static_cast<const uint16_t*>(a_lo);
   if (f16 && shape.pair >= 0 && skip_kblock < 0) {
     // segments at the online split's K ranges where each is one chain, else the unsplit form's chains
-    int chain = chain_blocks<Fp16x3>(1);
+    int chain = shape.chain;
     if (seg_splits > 1) chain = rank_blocks_of<Fp16x3>(a.K, seg_splits);
     if (chain > kChainBlocks) return SPL_EINVAL;
     return launch_pair(a, hi, lo, a_exp, shape.pair, chain);
@@ -2285,11 +2286,11 @@ int tc_uniform_splits(const Plan& p) {
   return p.tc.full_tiles > 0 ? 1 : p.tc.rest_splits;
 }
 
-spl_status run_tc_matched(const LinearArgs& a, int splits, int swap_ctas) {
+spl_status run_tc_matched(const LinearArgs& a, int splits, int swap_ctas, int chain) {
   if (swap_ctas > 0)  // the swapped kernel with the online runs; a width for all of M
     return run_tc_impl(a, -1, -1, 0, 0, 0, false, swap_width_index(a.M), swap_ctas);
   if (splits < 1 || splits > MAX_CLUSTER) return SPL_ESHAPE;
-  return run_tc_impl(a, -1, -1, 0, splits);
+  return run_tc_impl(a, -1, -1, 0, splits, 0, false, -1, 0, -1, nullptr, chain);
 }
 
 }  // namespace spl
@@ -2345,7 +2346,7 @@ extern "C" spl_status spl_test_tc_shape(int64_t M, int64_t K, int64_t N, int64_t
   if (!out || M <= 0 || K <= 0 || N <= 0 || seg_splits < 0 || seg_splits > MAX_CLUSTER) return SPL_EINVAL;
   const int sms = device_sm_count();
   const TcShape t =
-      seg_splits > 0 ? tc_bank_shape(M, K, N, (int)seg_splits, sms, true) : tc_shape(M, K, N, sms, true);
+      seg_splits > 0 ? tc_bank_shape(M, K, N, (int)seg_splits, sms, true, kChainBlocks) : tc_shape(M, K, N, sms, true);
   out[0] = t.pair >= 0 ? kPair[t.pair].bn : kVariant[t.v].bn;
   out[1] = t.pair >= 0 ? kPairRingKb : kVariant[t.v].rk;
   out[2] = t.full_tiles;

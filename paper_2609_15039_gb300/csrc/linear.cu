@@ -123,15 +123,17 @@ struct MatchedPlan {
   int64_t chunk_rows;  // decode kernel: rows per launch (<= 16)
   size_t ws;           // workspace bytes
   int swap_ctas;       // of the masked product (Plan)
+  int chain;           // of its unsplit tiles (TcShape)
 };
 
 MatchedPlan matched_plan(int64_t M, int64_t K, int64_t N, int64_t order_rows, spl_path resolved) {
-  MatchedPlan mp{false, 0, 1, K, M, 0, 0};
+  MatchedPlan mp{false, 0, 1, K, M, 0, 0, 0};
   const Plan online = make_plan(order_rows, K, N, resolved);
   mp.kernel = online.kernel;
   if (online.kernel == kKernelTc) {
     mp.splits = tc_uniform_splits(online);  // the bank runs its own launch shape; only the K-split order carries over
     mp.swap_ctas = online.swap_ctas;
+    mp.chain = online.tc.chain;
     if (mp.splits == 0) return mp;
     mp.ws = kCounterBytes + tc_asplit_bytes(M, K, resolved) + tc_partial_bytes(M, K, N, order_rows, resolved);
     mp.ok = true;
@@ -354,7 +356,7 @@ spl_status precompute_matched(float* C, const float* Nz, const spl_weight* A, co
     args.a_l16 = A->f16_lo;
     args.a_exp = A->f16_exp;
   }
-  if (mp.kernel == kKernelTc) return run_tc_matched(args, mp.splits, mp.swap_ctas);
+  if (mp.kernel == kKernelTc) return run_tc_matched(args, mp.splits, mp.swap_ctas, mp.chain);
   Plan p{};
   p.kernel = mp.kernel;
   p.splits = mp.splits;
