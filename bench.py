@@ -515,7 +515,7 @@ def run_llama_stack(args):
     roofline = {
         "bound": "tensor", "achieved": achieved, "peak": prod_peak, "unit": "TFLOP/s", "frac": achieved / prod_peak,
         "traffic": traffic,
-        "kernel": ("tc_persistent_kernel / tc_gemm_kernel (FP16X3 on tcgen05) with the fused unmask: " + what +
+        "kernel": ("tc_pair_kernel / tc_gemm_kernel (FP16X3 on tcgen05) with the fused unmask: " + what +
                    f"; {len(groups) * L} calls per step"),
         "flops_per_launch": call_flops_layer / len(groups), "avg_launch_us": 1e3 * prod_ms_layer / len(groups),
         "per_group": prod, "share_of_step": L * prod_ms_layer / ms,
