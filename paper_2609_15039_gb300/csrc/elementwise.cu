@@ -26,12 +26,18 @@ namespace {
 constexpr int kThreads = 256;
 
 // xt = x + eta (if xt), nout = eta (if nout).  n elements, nb = ceil(n/4) Philox blocks.
-// What bounds it, at 1e8 entries (800 MB, 120 us at the copy rate): without noise the loads in flight, so four blocks
-// a trip (two: 136 us, four: 120); the Laplace draw the wait for those loads too (149 -> 135 us); the Gaussian
-// draw the instructions (37 an entry, 2.7 to 2.9 issued a cycle of 4, 137 us with nothing read), where two
-// blocks a trip leave more registers (four: 154 us).  16 blocks an SM instead of 8 even out the end of the
-// grid (Gaussian 147 -> 143 us).
-template <int MECH>
+// PER blocks a trip, their loads issued first.  What bounds it, at 1e8 entries (800 MB, 120 us at the copy rate): without
+// noise and with Laplace the loads in flight, with Gaussian noise the instructions (37 an entry, 137 us with nothing
+// read).  Up to about 1e7 entries (kFew, kFewLaplace) few trips fill the grid, and a thread that has less than one trip takes its
+// entries one after another, so there 2 a trip and 8 blocks an SM; beyond, 4 and 16, which even out the end of the grid:
+//   entries                    2.07e6   5e6   7e6   1e7   2e7   1e8  (us)
+//   Laplace    2, 8 blocks       4.40  8.03  10.7  14.9  29.8   135
+//              4, 16             4.89  9.05  11.6  15.7  29.7   134
+//   Gaussian   2, 8              4.57  8.57  11.5  16.1  31.7   147
+//              4, 16             4.99  9.14  11.7  15.8  30.2   138
+//   eps = inf  2, 8              2.89  4.57  6.36  10.1  25.9   121
+//              4, 16             3.70  5.64  6.74   7.8  24.1   119
+template <int MECH, int PER>
 __global__ void __launch_bounds__(kThreads) noise_mask_kernel(float* xt, float* __restrict__ nout,
                                                               const float* x, int64_t n, float b,
                                                               const __grid_constant__ PhiloxKey key,
@@ -45,7 +51,6 @@ __global__ void __launch_bounds__(kThreads) noise_mask_kernel(float* xt, float* 
   const float4* x4 = reinterpret_cast<const float4*>(x);
   float4* xt4 = reinterpret_cast<float4*>(xt);
   float4* n4 = reinterpret_cast<float4*>(nout);
-  constexpr int PER = MECH == kGaussian ? 2 : 4;  // blocks per trip, their loads issued first
   for (; i + (PER - 1) * stride < nb_full; i += PER * stride) {
     float4 xv[PER];
 #pragma unroll
@@ -392,15 +397,17 @@ spl_status launch_noise_mask(float* xt, float* nout, const float* x, int64_t n, 
                              spl_mech mech, spl_rng rng, cudaStream_t stream) {
   if ((reinterpret_cast<uintptr_t>(rng.offset_dev) & 7u) != 0) return SPL_EALIGN;
   const float b = std::isinf(eps) ? 0.0f : (float)(sensitivity / eps);
-  const int grid = grid_for(ceil_div(n, 4), 16);
   const PhiloxKey key = make_philox_key(rng.seed, rng.stream_id);
-  if (b == 0.0f) {
-    return launch_pdl(noise_mask_kernel<kZero>, dim3(grid), dim3(kThreads), 0, stream, xt, nout, x, n, b, key, rng.offset, rng.offset_dev);
-  } else if (mech == SPL_MECH_LAPLACE) {
-    return launch_pdl(noise_mask_kernel<kLaplace>, dim3(grid), dim3(kThreads), 0, stream, xt, nout, x, n, b, key, rng.offset, rng.offset_dev);
-  } else {
-    return launch_pdl(noise_mask_kernel<kGaussian>, dim3(grid), dim3(kThreads), 0, stream, xt, nout, x, n, b, key, rng.offset, rng.offset_dev);
-  }
+  auto launch = [&](auto small, auto large, int64_t few) {
+    const bool is_small = n < few;
+    return launch_pdl(is_small ? small : large, dim3(grid_for(ceil_div(n, 4), is_small ? 8 : 16)), dim3(kThreads), 0, stream,
+                      xt, nout, x, n, b, key, rng.offset, rng.offset_dev);
+  };
+  // where 4 blocks a trip and 16 an SM start to win (the table at the kernel)
+  constexpr int64_t kFew = int64_t(1) << 23, kFewLaplace = int64_t(1) << 24;
+  if (b == 0.0f) return launch(noise_mask_kernel<kZero, 2>, noise_mask_kernel<kZero, 4>, kFew);
+  if (mech == SPL_MECH_LAPLACE) return launch(noise_mask_kernel<kLaplace, 2>, noise_mask_kernel<kLaplace, 4>, kFewLaplace);
+  return launch(noise_mask_kernel<kGaussian, 2>, noise_mask_kernel<kGaussian, 4>, kFew);
 }
 
 }  // namespace
