@@ -437,12 +437,17 @@ __device__ __forceinline__ void reduce_store(float* red, bool ragged, int r0, in
 // Rows r0..r1 of the staged sums minus C, stored, where the output's rows are no whole 16-byte units (N % 4 != 0):
 // by single elements, a warp's lanes along a row, so that C and the output move in whole lines, and P elements of C
 // in flight per thread.  (Four neighbours a thread, each C loaded where it was subtracted, took 24.1 us for 128 rows
-// of 3072 by 5121 where this takes 22.4, and 22.9 for 61 of 2560 by 6143 where this takes 21.2.)
+// of 3072 by 5121 where this takes 23.6, and 52.0 for 61 of 2560 by 6143 unsplit, 128 wide, where this takes 35.1.)
+// Of a width that is a power of two the last trip ends where the block's elements do: without that a CTA of a split
+// computed up to twice its elements (1000 x 512 by 9001, 256 wide, 4 ways 138 us, 127 so; 5 ways 183, 162).  Of others
+// it does not: the early end keeps the compiler from sharing the divisions among the P elements (192 wide, unsplit 75
+// us, 81 so; 40 x 2048 by 9999, 224 wide, 3 ways 25 us, 28 so).
 template <int BN>
 __device__ __forceinline__ void store_ragged(const float* red, int r0, int r1, int64_t m0, int64_t n0, int64_t M,
                                              int64_t N, const float* __restrict__ C, float* __restrict__ out,
                                              int64_t c_rows) {
-  constexpr int RS = BN + 4, P = 32;
+  constexpr bool kStop = (BN & (BN - 1)) == 0;
+  constexpr int RS = BN + 4, P = kStop ? 44 : 32;
   const int cols = (int)std::min<int64_t>(BN, N - n0);
   const int rows = (int)std::min<int64_t>(r1, M - m0) - r0;
   const int c_end = C && m0 < c_rows ? (int)std::min<int64_t>(r1, c_rows - m0) - r0 : 0;  // rows below it subtract C
@@ -451,11 +456,13 @@ __device__ __forceinline__ void store_ragged(const float* red, int r0, int r1, i
     float cc[P];
 #pragma unroll
     for (int u = 0; u < P; ++u) {
+      if (kStop && base + u * THREADS >= rows * BN) break;
       const int r = (base + u * THREADS) / BN, c = (base + u * THREADS) % BN;
       cc[u] = c < cols && r < rows && r < c_end ? __ldcs(C + origin + r * N + c) : 0.f;
     }
 #pragma unroll
     for (int u = 0; u < P; ++u) {
+      if (kStop && base + u * THREADS >= rows * BN) break;
       const int r = (base + u * THREADS) / BN, c = (base + u * THREADS) % BN;
       if (c >= cols || r >= rows) continue;
       const float v = red[(r0 + r) * RS + c];
