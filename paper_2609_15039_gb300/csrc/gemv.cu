@@ -123,27 +123,46 @@ struct KernelNoise {
   uint64_t delta;
 };
 
-// The masked instances of a row count keep as many blocks an SM as the unmasked one, for which the plan sizes the
-// grid (3, 2 and 3 at 1, 2 and 4 rows), and the registers that the two buffers of W need.  Left alone, the compiler
-// took 64 to 94 registers for them: instances of 64 held fewer loads in flight, and one row at eps = inf got 2
-// blocks of the 3, a second wave.  us a step of two Llama layers without Down, before and now:
+// The masked instances come in two forms, MANY for grids of many waves (many_waves: where the line lies).
+//
+// Few waves: as many blocks an SM as the unmasked instance, for which the plan sizes the grid (3, 2 and 3 at 1, 2 and 4
+// rows), and the registers that the two buffers of W need.  Left alone, the compiler took 64 to 94 registers: instances
+// of 64 held fewer loads in flight, and one row at eps = inf got 2 blocks of the 3, a second wave.  us a step of two
+// Llama layers without Down, before and now:
 //   rows                  1     2     4     1 + 1   2 + 2 (a step's rows and the next cycle's)
 //   Laplace   before  115.6 114.2 123.4   113.3   122.8
 //             now     110.9 112.9 122.5   111.5   122.2
 //   Gaussian  before  107.1 132.1 133.3   131.5   132.5
 //             now     107.0 112.3 121.6   111.8   121.0
 //   eps = inf before  133.0 113.2 118.9   111.5   116.7
-//             now     106.6 109.4 118.6   108.4   116.8
-constexpr int masked_blocks(int mt) { return mt == 2 ? 2 : mt == 4 ? 3 : 0; }  // 0: the compiler's choice already
+//             now     107.5 109.4 119.0   108.3   116.8
+//
+// Many waves: the registers that the compiler takes for staging row by row (two rows' draws side by side), 64 and 4
+// blocks an SM at 4 rows (and 1 row with noise): blocks follow one another, and more of them cover a block's start and
+// end.  us, few / many:
+//   K x N              6784 x 20976   2048 x 32768   3072 x 128256
+//   4 rows, Laplace      98.7 / 94.9    49.5 / 45.7     245 / 241
+//   4 rows, Gaussian     97.3 / 93.5    48.2 / 45.5     244 / 239
+//   4 rows, eps = inf    96.7 / 89.3    50.7 / 44.2     246 / 233
+//   2 rows, eps = inf    94.6 / 87.5                    248 / 237
+//   1 row, Laplace                                      238 / 232
+constexpr int masked_blocks(int mt, int mask, bool many) {  // 0: the compiler's choice does
+  if (mask == kNoMask) return 0;
+  return many ? 0 : mt == 2 ? 2 : mt == 4 ? 3 : 0;
+}
 // One pointer to the lane's rows and their distance instead of a pointer a row: 8 registers.  (One row with Gaussian
 // noise is 109.1 us so, 107.0 with the pointers.)
-constexpr bool one_pointer(int mt, int mask) { return mask != kNoMask && !(mt == 1 && mask == kGaussian); }
+constexpr bool one_pointer(int mt, int mask, bool many) {
+  return mask != kNoMask && !many && !(mt == 1 && mask == kGaussian);
+}
 // W's first steps are fetched before the wait: where no noise is drawn meanwhile, which needs the registers (eps = inf
 // 109 -> 106 us at one row and 112 -> 109 at two, but 118 -> 122 at four).
-constexpr bool early_weights(int mt, int mask) { return mask == kNoMask || (mask == kZero && mt <= 2); }
+constexpr bool early_weights(int mt, int mask, bool many) {
+  return mask == kNoMask || (mask == kZero && mt <= 2 && !many);
+}
 
-template <int MT, int MASK>
-__global__ void __launch_bounds__(THREADS, MASK == kNoMask ? 0 : masked_blocks(MT))
+template <int MT, int MASK, bool MANY>
+__global__ void __launch_bounds__(THREADS, masked_blocks(MT, MASK, MANY))
 gemv_kernel(float* __restrict__ out, const float* __restrict__ X, const float* __restrict__ W,
             const float* __restrict__ C, float* __restrict__ part, unsigned int* __restrict__ counters, int M,
             int64_t K, int64_t N, int ks, int splits, int prefetch_lines, const __grid_constant__ KernelNoise nz,
@@ -168,7 +187,7 @@ gemv_kernel(float* __restrict__ out, const float* __restrict__ X, const float* _
   }
   const float* const w0 = W + row0 * K + k0 + kl;
   const int n_left = (int)std::max<int64_t>(0, std::min<int64_t>(N - row0, 4 * RQ));
-  constexpr bool kOne = one_pointer(MT, MASK), kEarly = early_weights(MT, MASK);
+  constexpr bool kOne = one_pointer(MT, MASK, MANY), kEarly = early_weights(MT, MASK, MANY);
   auto row_in = [&](int r) { return kOne ? 4 * r < n_left : valid[r]; };
   auto row_at = [&](int r) { return kOne ? w0 + (int64_t)(4 * r) * K : wp[r]; };
 
@@ -215,6 +234,41 @@ gemv_kernel(float* __restrict__ out, const float* __restrict__ X, const float* _
 #pragma unroll
       for (int m = 0; m < MT; ++m)
         for (int q = threadIdx.x; q < q_row; q += THREADS) xs[m * q_row + q] = x4(m, q);
+    }
+  } else if constexpr (MASK != kNoMask && MANY) {
+    // as the list below, the rows in turn
+    const uint64_t off = nz.offset + (nz.offset_dev ? *nz.offset_dev : 0ull);
+    const bool write_xt = blockIdx.x == 0;
+    auto xt_at = [&](int m, int q) {
+      return write_xt && m < M && q < q_len ? reinterpret_cast<float4*>(nz.xt + (int64_t)m * K + k0) + q : nullptr;
+    };
+    // dst: where X~ goes, null for nowhere (4 rows: made outside it leaves 64 registers, inside 78; at 1 row the reverse)
+    auto x4 = [&](int m, int q, float4* dst) -> float4 {
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (m < M && q < q_len) {
+        const bool own = m < nz.x_rows;
+        const int64_t mr = own ? m : m - nz.x_rows;
+        if (own) v = __ldg(reinterpret_cast<const float4*>(X + (int64_t)m * K + k0) + q);
+        const float4 e = draw_block<MASK>((uint64_t)((mr * K + k0) >> 2) + (uint64_t)q + off + (own ? 0ull : nz.delta),
+                                          nz.key, nz.b);
+        v = own ? add4(v, e) : e;
+        if (MT >= 4 ? dst != nullptr : write_xt)
+          __stcs(MT >= 4 ? dst : reinterpret_cast<float4*>(nz.xt + (int64_t)m * K + k0) + q, v);
+      }
+      return v;
+    };
+    if constexpr (MT >= 4) {  // rows 2p, 2p + 1 interleaved
+#pragma unroll
+      for (int p = 0; p < MT / 2; ++p)
+        for (int q = threadIdx.x; q < q_row; q += THREADS) {
+          const float4 a = x4(2 * p, q, xt_at(2 * p, q)), b = x4(2 * p + 1, q, xt_at(2 * p + 1, q));
+          *reinterpret_cast<float4*>(xsf + pair_off(p, ksp, q, 0)) = make_float4(a.x, b.x, a.y, b.y);
+          *reinterpret_cast<float4*>(xsf + pair_off(p, ksp, q, 1)) = make_float4(a.z, b.z, a.w, b.w);
+        }
+    } else {
+#pragma unroll
+      for (int m = 0; m < MT; ++m)
+        for (int q = threadIdx.x; q < q_row; q += THREADS) xs[m * q_row + q] = x4(m, q, nullptr);
     }
   } else {
     // Fused mask: X~ = fl32(X + eta), eta of element (m, k) being lane k % 4 of Philox block (m K + k) / 4 + offset,
@@ -396,12 +450,13 @@ gemv_kernel(float* __restrict__ out, const float* __restrict__ X, const float* _
     float s = 0.f;
     // 8 slices' loads in flight, added in order (one at a time they were a latency each: 8 rows of Llama Q|K|V
     // 18.7 -> 17.5 us, one row of O 9.8 -> 9.1 us, with one fence a block instead of one a thread)
-    for (int sp = 0; sp < splits; sp += 8) {
-      float v[8];
+    constexpr int kAtOnce = MANY && MT == 1 && MASK == kZero ? 16 : 8;  // 16: 3 blocks an SM there instead of 2
+    for (int sp = 0; sp < splits; sp += kAtOnce) {
+      float v[kAtOnce];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) v[i] = sp + i < splits ? __ldcg(part + (int64_t)(sp + i) * M * N + o) : 0.f;
+      for (int i = 0; i < kAtOnce; ++i) v[i] = sp + i < splits ? __ldcg(part + (int64_t)(sp + i) * M * N + o) : 0.f;
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
+      for (int i = 0; i < kAtOnce; ++i)
         if (sp + i < splits) s = sp + i == 0 ? v[i] : __fadd_rn(s, v[i]);
     }
     out[o] = (C && m < c_rows) ? __fsub_rn(s, c) : s;
@@ -411,8 +466,21 @@ gemv_kernel(float* __restrict__ out, const float* __restrict__ X, const float* _
 
 int padded_m(int64_t M) { return M <= 1 ? 1 : M <= 2 ? 2 : M <= 4 ? 4 : M <= 8 ? 8 : 16; }
 
-template <int MT, int MASK = kNoMask>
-void* kernel_ptr() { return reinterpret_cast<void*>(gemv_kernel<MT, MASK>); }
+template <int MT, int MASK = kNoMask, bool MANY = false>
+void* kernel_ptr() { return reinterpret_cast<void*>(gemv_kernel<MT, MASK, MANY>); }
+
+// Whether a masked call of this many waves (of the blocks that the plan counts on) takes the MANY form.  At 4 rows F = the
+// few-waves form and M = the other cross between 1.9 waves (4096 x 11008: F 33.9, M 34.6 us with Laplace noise, 32.5
+// and 36.0 at eps = inf) and 2.3 (2048 x 32768: F 49.5, M 45.7); one row at eps = inf already about one wave (3072 x
+// 16384, 0.84: F 34.3, M 33.8; 8192 x 3072, 1.00: 18.0 and 17.2; but 1152 x 5003, 0.79: 6.4 and 7.1); two rows with
+// noise nowhere (6784 x 20976, 2.7: F 92.7, M 93.6; 3072 x 128256, 6.6: 246 and 249).  One row with Laplace noise takes M
+// also where the grid leaves most of the chip idle (1024 x 1024, 0.14: F 4.7, M 4.1; 512 x 8192, 0.56: 6.5 and 6.0; but 3072
+// x 5120, 0.88: 12.3 and 13.4).
+bool many_waves(int mt, int mask, double waves) {
+  if (mt == 2 && mask != kZero) return false;
+  if (mt == 1 && mask == kLaplace && waves < 0.6) return true;
+  return waves > (mt == 1 && mask == kZero ? 0.82 : 2.0);
+}
 
 void* kernel_for(int mt) {
   switch (mt) {
@@ -435,7 +503,10 @@ bool smem_attr_set() {
     void* const kernels[] = {kernel_ptr<1>(), kernel_ptr<2>(), kernel_ptr<4>(), kernel_ptr<8>(), kernel_ptr<16>(),
                              kernel_ptr<1, kZero>(), kernel_ptr<2, kZero>(), kernel_ptr<4, kZero>(),
                              kernel_ptr<1, kLaplace>(), kernel_ptr<2, kLaplace>(), kernel_ptr<4, kLaplace>(),
-                             kernel_ptr<1, kGaussian>(), kernel_ptr<2, kGaussian>(), kernel_ptr<4, kGaussian>()};
+                             kernel_ptr<1, kGaussian>(), kernel_ptr<2, kGaussian>(), kernel_ptr<4, kGaussian>(),
+                             kernel_ptr<1, kZero, true>(), kernel_ptr<2, kZero, true>(), kernel_ptr<4, kZero, true>(),
+                             kernel_ptr<1, kLaplace, true>(), kernel_ptr<4, kLaplace, true>(),
+                             kernel_ptr<1, kGaussian, true>(), kernel_ptr<4, kGaussian, true>()};
     for (void* k : kernels)
       if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kXsBytes) != cudaSuccess) {
         cudaGetLastError();
@@ -446,7 +517,7 @@ bool smem_attr_set() {
   return true;
 }
 
-template <int MT, int MASK = kNoMask>
+template <int MT, int MASK = kNoMask, bool MANY = false>
 spl_status launch(const LinearArgs& a, const Plan& p, float* part, unsigned int* counters,
                   const KernelNoise& nz = KernelNoise{}) {
   if (!smem_attr_set()) return SPL_ECUDA;
@@ -455,18 +526,8 @@ spl_status launch(const LinearArgs& a, const Plan& p, float* part, unsigned int*
   // L2 budget of the early prefetch: about 32 MB over the whole grid, in 128-byte lines per row
   const int64_t rows = (int64_t)grid.x * rows_per_block(MT) * p.splits;
   const int lines = (int)std::min<int64_t>(p.k_per_split / kStep, ((int64_t(32) << 20) / std::max<int64_t>(rows, 1)) >> 7);
-  return launch_pdl(gemv_kernel<MT, MASK>, grid, dim3(THREADS), smem, a.stream, a.out, a.a, a.w, a.c, part, counters,
+  return launch_pdl(gemv_kernel<MT, MASK, MANY>, grid, dim3(THREADS), smem, a.stream, a.out, a.a, a.w, a.c, part, counters,
                     (int)a.M, a.K, a.N, (int)p.k_per_split, p.splits, lines, nz, (int)a.c_rows);
-}
-
-template <int MASK>
-spl_status launch_masked(const LinearArgs& a, const Plan& p, float* part, unsigned int* counters,
-                         const KernelNoise& nz) {
-  switch (padded_m(a.M)) {
-    case 1: return launch<1, MASK>(a, p, part, counters, nz);
-    case 2: return launch<2, MASK>(a, p, part, counters, nz);
-    default: return launch<4, MASK>(a, p, part, counters, nz);
-  }
 }
 
 // Resident blocks per SM of the decode kernel for MT rows and a K-slice of ks (cached).
@@ -490,7 +551,23 @@ int blocks_per_sm(int mt, int64_t ks) {
   return v;
 }
 
-// The instance for `mask` (kNoMask, or a mechanism) at a padded row count, null where there is none.
+template <int MASK>
+spl_status launch_masked(const LinearArgs& a, const Plan& p, float* part, unsigned int* counters,
+                         const KernelNoise& nz) {
+  const int mt = padded_m(a.M);
+  const double slots = (double)device_sm_count() * blocks_per_sm(mt, p.k_per_split);
+  const bool many = many_waves(mt, MASK, (double)(ceil_div(a.N, rows_per_block(mt)) * p.splits) / slots);
+  if (mt == 1)
+    return many ? launch<1, MASK, true>(a, p, part, counters, nz) : launch<1, MASK>(a, p, part, counters, nz);
+  if (mt == 2) {
+    if constexpr (MASK == kZero)
+      if (many) return launch<2, MASK, true>(a, p, part, counters, nz);
+    return launch<2, MASK>(a, p, part, counters, nz);
+  }
+  return many ? launch<4, MASK, true>(a, p, part, counters, nz) : launch<4, MASK>(a, p, part, counters, nz);
+}
+
+// The instance for `mask` (kNoMask, or a mechanism) and few waves at a padded row count, null where there is none.
 void* instance_for(int mt, int mask) {
   if (mask == kNoMask) return kernel_for(mt);
   if (mt > kGemvMaskMaxM || mask < kLaplace || mask > kZero) return nullptr;
